@@ -123,6 +123,10 @@ struct rlgl_ctx {
     int grid_power = 0;
     int* hubs = nullptr;  // hub table of the push (kHubSlots ids, -1 empty), null when none
     int n_hubs = 0;
+    int hub1 = -1;        // the hub when there is one
+    int* deg = nullptr;      // links of each row
+    void* f_list = nullptr;  // the phase kernels' f_eoff and f_base; the sweep's list of green rows
+    void* pieces = nullptr;  // pieces of the long green rows of a move (sweep)
     // profiling
     int profiling = 0;
     std::vector<ProfEv> prof;
@@ -240,6 +244,12 @@ static rlgl_status dalloc(rlgl_ctx* ctx, P** p, size_t count) {
 
 static void dfree(rlgl_ctx* ctx, void* p) {
     if (p) cudaFreeAsync(p, ctx->stream);
+}
+
+// Bytes of the table of long green rows' pieces: at most one piece per
+// kHubRow links, and one more per row of more than kHubRow.
+static size_t pieces_bytes(long long nnz, size_t cash) {
+    return (size_t)(2 * (nnz / kHubRow) + 1) * (cash == 4 ? sizeof(Piece<float>) : sizeof(Piece<double>));
 }
 
 static size_t cash_size(const rlgl_ctx* ctx) {
@@ -421,12 +431,13 @@ static rlgl_status enqueue_pull(Launch L) {
 // A persistent kernel (rlgl_sweep.cuh, rlgl_power.cuh): one cooperative
 // launch of `grid` blocks, never more than fit on the device at once.
 template <typename T>
-static rlgl_status launch_coop(rlgl_ctx* ctx, int grid, void (*kernel)(SweepArgs<T>), const SweepArgs<T>& a) {
+static rlgl_status launch_coop(rlgl_ctx* ctx, int grid, int threads, size_t smem, void (*kernel)(SweepArgs<T>),
+                               const SweepArgs<T>& a) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = 0;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = ctx->stream;
     cudaLaunchAttribute attr[1];
     memset(attr, 0, sizeof attr);
@@ -451,10 +462,12 @@ static SweepArgs<T> sweep_args(rlgl_ctx* ctx, const Conds& cd) {
     a.mt = (T*)ctx->mt;
     a.mt2 = (T*)ctx->hsrc;  // free while no re-derivation runs
     a.facc = (T*)ctx->f_m;  // the power sweep clears it at every launch
-    a.f_eoff = ctx->f_eoff;
-    a.f_base = ctx->f_base;
-    a.f_m = (T*)ctx->f_m;
-    a.chunk_row = ctx->chunk_row;
+    // (f_list: f_eoff and f_base, one after the other)
+    a.deg = ctx->deg;
+    a.list = (Green<T>*)ctx->f_list;
+    a.pieces = (Piece<T>*)ctx->pieces;
+    a.n_hubs = ctx->n_hubs;
+    a.hub1 = ctx->hub1;
     a.col = ctx->col;
     a.w = ctx->w;
     a.t_ptr = ctx->t_ptr;
@@ -483,9 +496,9 @@ static rlgl_status enqueue_sweep(Launch L, const Conds& cd) {
     rlgl_ctx* ctx = L.ctx;
     const SweepArgs<T> a = sweep_args<T>(ctx, cd);
     if (ctx->has_w)
-        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_sweep, k_sweep<T, true>, a))));
+        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_sweep, kSweepThreads, sizeof(SweepSmem<T>), k_sweep<T, true>, a))));
     else
-        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_sweep, k_sweep<T, false>, a))));
+        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_sweep, kSweepThreads, sizeof(SweepSmem<T>), k_sweep<T, false>, a))));
     return RLGL_OK;
 }
 
@@ -495,9 +508,9 @@ static rlgl_status enqueue_power(Launch L, const Conds& cd) {
     rlgl_ctx* ctx = L.ctx;
     const SweepArgs<T> a = sweep_args<T>(ctx, cd);
     if (ctx->has_w)
-        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_power, k_power<T, true>, a))));
+        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_power, kThreads, 0, k_power<T, true>, a))));
     else
-        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_power, k_power<T, false>, a))));
+        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_power, kThreads, 0, k_power<T, false>, a))));
     return RLGL_OK;
 }
 
@@ -592,17 +605,21 @@ static int bsweep_fit(rlgl_ctx* ctx, int bt) {
 // Blocks of the sweep: all that fit on the device at once (the occupancy of
 // the instantiation this context uses), fewer for a small chain, where each
 // block still gets at least one block-iteration of nodes.
-template <typename T>
-static int sweep_fit(rlgl_ctx* ctx) {
+template <typename T, bool kHasW>
+static int sweep_fit_t() {
     int nb = 0;
-    cudaError_t e = ctx->has_w
-                        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sweep<T, true>, kThreads, 0)
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sweep<T, false>, kThreads, 0);
-    if (e != cudaSuccess) {
+    constexpr int smem = (int)sizeof(SweepSmem<T>);
+    if (cudaFuncSetAttribute(k_sweep<T, kHasW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sweep<T, kHasW>, kSweepThreads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return nb;
+}
+
+template <typename T>
+static int sweep_fit(rlgl_ctx* ctx) {
+    return ctx->has_w ? sweep_fit_t<T, true>() : sweep_fit_t<T, false>();
 }
 
 static int sweep_grid(rlgl_ctx* ctx) {
@@ -909,19 +926,21 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
     TRY(dalloc(ctx, &ctx->y, (size_t)n));
     TRY(dalloc(ctx, &ctx->hsrc, (size_t)n));
     TRY(dalloc(ctx, &ctx->colsum, (size_t)n));
-    TRY(dalloc(ctx, &ctx->f_eoff, (size_t)n));
-    TRY(dalloc(ctx, &ctx->f_base, (size_t)n));
+    TRY(dalloc_bytes(ctx, &ctx->f_list, 2 * (size_t)n * sizeof(long long)));
+    ctx->f_eoff = (long long*)ctx->f_list;
+    ctx->f_base = ctx->f_eoff + n;
+    TRY(dalloc(ctx, &ctx->deg, (size_t)n));
     TRY(dalloc_bytes(ctx, &ctx->f_m, (size_t)n * cs));
     TRY(dalloc(ctx, &ctx->chunk_row, (size_t)(nnz / kPushChunk + 2)));
     TRY(dalloc(ctx, &ctx->part, (size_t)(4 * kMaxGrid + 8)));
+    TRY(dalloc_bytes(ctx, &ctx->pieces, pieces_bytes(nnz, cs)));
     TRY(dalloc(ctx, &ctx->err, 1));
     TRY(dalloc(ctx, &ctx->log, (size_t)kLogCap));
     TRY(dalloc(ctx, &ctx->st, 1));
     TRY(dalloc(ctx, &ctx->sw, 1));
-    // the sweep reads slot fields in 16-byte pairs and stages the cash, 1/d
-    // and row offsets with 16-byte copies (pool allocations are aligned far
-    // beyond that)
-    if ((((uintptr_t)ctx->sw | (uintptr_t)ctx->c | (uintptr_t)ctx->ideg | (uintptr_t)ctx->row_ptr) & 15u) != 0)
+    // the sweep reads slot fields in 16-byte pairs (pool allocations are
+    // aligned far beyond that)
+    if ((((uintptr_t)ctx->sw | (uintptr_t)ctx->pieces | (uintptr_t)ctx->f_list) & 15u) != 0)
         return fail(ctx, RLGL_ENOMEM, "device buffers not 16-byte aligned");
     ctx->host_st = static_cast<DevState*>(pin_get());
     if (!ctx->host_st) return fail(ctx, RLGL_ENOMEM, "pinned host allocation failed");
@@ -953,7 +972,7 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
     k_row_scale<<<gn, kThreads, 0, ctx->stream>>>(
         ctx->row_ptr, ctx->w, n, ctx->s, ctx->sf,
         prec == RLGL_MIXED ? (float*)ctx->ideg : nullptr,
-        prec == RLGL_MIXED ? nullptr : (double*)ctx->ideg, ctx->chunk_row, ctx->err);
+        prec == RLGL_MIXED ? nullptr : (double*)ctx->ideg, ctx->deg, ctx->chunk_row, ctx->err);
     CKL(ctx);
     if (ctx->has_w) {
         const long long max_long = nnz / kLongRowW + 1;  // rows longer than kLongRowW
@@ -1046,6 +1065,7 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
         }
         ctx->n_hubs = got;
         if (got) {
+            if (got == 1) ctx->hub1 = *std::max_element(tab, tab + kHubSlots);  // the others are -1
             TRY(dalloc(ctx, &ctx->hubs, kHubSlots));
             CK(ctx, cudaMemcpyAsync(ctx->hubs, tab, sizeof tab, cudaMemcpyHostToDevice, ctx->stream));
         }
@@ -1990,10 +2010,11 @@ int64_t rlgl_footprint(int64_t n, int64_t nnz, int32_t weighted, rlgl_precision 
     const int64_t nwtiles = (n + nnz + witems - 1) / witems;
     int64_t b = 0;
     b += 2 * ((n + 1) * 8 + nnz * 4 + (weighted ? nnz * 4 : 0));  // CSR and CSC
-    b += n * (8 + (prec == RLGL_MIXED ? 4 : 0) + cs);                // s, sf, 1/deg
+    b += n * (8 + (prec == RLGL_MIXED ? 4 : 0) + cs + 4);            // s, sf, 1/deg, deg
     b += 2 * (ntiles + 1) * 8 + 2 * (nwtiles + 1) * 8;               // merge-path tiles (block, warp)
     b += n * (cs + 8 + cs + 8 + 8 + 8 + 8 + cs + 8);                 // c H mt y hsrc f_eoff f_base f_m colsum
     b += (nnz / kPushChunk + 2) * 4;                                 // chunk index
+    b += (int64_t)pieces_bytes(nnz, (size_t)cs);                    // long rows' pieces
     b += (4 * kMaxGrid + 8) * 8 + 8 + (int64_t)kLogCap * (int64_t)sizeof(MoveRecord) +
          (int64_t)sizeof(DevState) + (int64_t)sizeof(SweepState);
     if (n_chains > 1) b += (n_chains + 1) * 8 + n * 4 + n_chains * ((int64_t)sizeof(ChainState) + 16);
@@ -2033,9 +2054,10 @@ void rlgl_destroy(rlgl_ctx* ctx) {
     void* dev[] = {ctx->row_ptr, ctx->col, ctx->w, ctx->s, ctx->sf, ctx->ideg, ctx->t_ptr, ctx->t_src, ctx->t_w,
                    ctx->tile_r, ctx->tile_e, ctx->wtile_r, ctx->wtile_e, ctx->c, ctx->H, ctx->mt, ctx->y, ctx->hsrc, ctx->c0,
                    ctx->colsum,
-                   ctx->f_eoff, ctx->f_base, ctx->f_m, ctx->chunk_row, ctx->part, ctx->masks,
+                   ctx->f_list, ctx->deg, ctx->f_m, ctx->chunk_row, ctx->part, ctx->masks,
                    ctx->err, ctx->log, ctx->st, ctx->sw, ctx->node_ptr, ctx->chain_of, ctx->cs,
-                   ctx->bsums, ctx->ct_off, ctx->ct_r, ctx->ct_e, ctx->grp, ctx->bq, ctx->q_next, ctx->hubs};
+                   ctx->bsums, ctx->ct_off, ctx->ct_r, ctx->ct_e, ctx->grp, ctx->bq, ctx->q_next, ctx->hubs,
+                   ctx->pieces};
     for (void* p : dev)
         dfree(ctx, p);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);

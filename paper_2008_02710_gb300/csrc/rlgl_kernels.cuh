@@ -35,6 +35,8 @@ constexpr int kNodesPerIter = kThreads * kNodesPerThread;
 constexpr int kPushChunk = 1024;      // edges per push chunk
 constexpr int kMpIpt = 8;             // merge-path items per thread
 constexpr int kMpItems = kThreads * kMpIpt;  // merge-path items (rows + edges) per tile
+constexpr int kShortRow = 64;         // sweep: longest row a warp pushes together with others
+constexpr int kHubRow = 512;          // sweep: longest row that its block pushes; longer ones go to all blocks in such pieces
 constexpr int kCountBits = 27;        // frontier reservation: (edges << 27) | count
 constexpr int kRadixBits = 11;
 constexpr int kRadixBins = 1 << kRadixBits;
@@ -1310,7 +1312,7 @@ __device__ __forceinline__ TV block_segscan(long long key, TV val, long long* s_
 // Shared memory of the merge-path tile loop.
 // Merge-path items per thread for a block of kBT threads: a tile is
 // kBT * mp_ipt(kBT) items (2048 for 256 threads).
-__host__ __device__ constexpr int mp_ipt(int kBT) { return kBT >= 512 ? 4 : kMpIpt; }
+__host__ __device__ constexpr int mp_ipt(int kBT) { return kBT >= 1024 ? 2 : (kBT >= 512 ? 4 : kMpIpt); }
 
 template <typename TV, int kBT = kThreads>
 struct PullSmem {
@@ -1739,11 +1741,12 @@ constexpr long long kLongRowW = 65536;
 __global__ void k_row_scale(const long long* __restrict__ row_ptr, const float* __restrict__ w,
                             long long n, double* __restrict__ s, float* __restrict__ sf,
                             float* __restrict__ idegf, double* __restrict__ idegd,
-                            int* __restrict__ long_rows, unsigned int* __restrict__ n_long) {
+                            int* __restrict__ deg, int* __restrict__ long_rows, unsigned int* __restrict__ n_long) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         long long a = row_ptr[i], b = row_ptr[i + 1];
         const double id = 1.0 / (double)(b - a);
+        deg[i] = (int)(b - a);
         if (idegf) idegf[i] = (float)id;
         if (idegd) idegd[i] = id;
         double sum;

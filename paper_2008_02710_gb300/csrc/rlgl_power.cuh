@@ -422,8 +422,6 @@ __device__ __forceinline__ void power_publish(PowAcc<T>& acc, SweepSlot* sl, T* 
     acc.a = acc.s = acc.m = acc.ma = T(0);
 }
 
-__device__ __forceinline__ int rot3(int q) { return q == 2 ? 0 : q + 1; }
-
 template <typename T, bool kHasW>
 __global__ void __launch_bounds__(kThreads, kPowerMinBlocks) k_power(SweepArgs<T> A) {
     DevState* st = A.st;
@@ -607,20 +605,20 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks) k_power(SweepArgs<T
 
         // ----------------------------------------------------------- move
         SweepSlot* nsl = &sw->slot[rot3(sc.p)];  // this move's sums and tile counter
-        if (lead) sc.ts[0] = globaltimer();
+        if (lead) sc.ts[0][0] = globaltimer();
         power_tiles<T, kHasW>(A, mt_cur, mt_nxt, sm[threadIdx.x >> 5], &nsl->chunk_next, acc);
-        if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts + 1 : nullptr))
+        if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts[0] + 1 : nullptr))
             break;
         power_split_rows<T>(A, mt_nxt, acc);
         power_publish<T>(acc, nsl, tscratch);
-        if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts + 3 : nullptr))
+        if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts[0] + 3 : nullptr))
             break;
         if (lead) {
             MoveRecord* rec = A.log + ((sc.moves - 1) % kLogCap);
             // the move's work (pull, then the split rows) and the waits at its
             // two barriers (slots 4 and 5)
-            rec->phase_us[4] = (float)((sc.ts[1] - sc.ts[0]) + (sc.ts[3] - sc.ts[2])) * 1e-3f;
-            rec->phase_us[5] = (float)((sc.ts[2] - sc.ts[1]) + (sc.ts[4] - sc.ts[3])) * 1e-3f;
+            rec->phase_us[4] = (float)((sc.ts[0][1] - sc.ts[0][0]) + (sc.ts[0][3] - sc.ts[0][2])) * 1e-3f;
+            rec->phase_us[5] = (float)((sc.ts[0][2] - sc.ts[0][1]) + (sc.ts[0][4] - sc.ts[0][3])) * 1e-3f;
         }
         {
             T* t = mt_cur;

@@ -3,19 +3,28 @@
 // costs three grid barriers (two with the stale threshold) instead of three
 // to four kernel launches, their drain and their serial last-block tails.
 //
-// Every block runs every phase of a move on its share of the work:
-//   stats   : its slice of the nodes; block sums go to one FP64 atomic per
-//             statistic in the move's slot;
+// One block of 1024 threads an SM owns a contiguous span of the nodes; a move is
+//   stats   : the statistics of its nodes' cash; block sums go to one FP64
+//             atomic per statistic in the move's slot;
 //   barrier ; every block reads the totals and takes the same decisions
 //             (stop, re-derivation, theta) from the same numbers;
 //   [top-k] : TOPFRAC only: the radix passes of the exact k-th largest |C|,
 //             each a count over the block's nodes and a barrier;
-//   select  : its node ranges, staged in shared memory by asynchronous
-//             copies (the same compaction as k_select);
-//   barrier ; every block reads the frontier size and picks push or pull;
-//   push    : its share of the frontier's edge chunks, or
+//   select  : its green nodes give up their cash and are listed;
+//   barrier ; every block reads the move's links and picks push or pull;
+//   push    : its own green rows, and a share of the pieces of the longest
+//             rows of all blocks, or
 //   pull    : its share of the merge-path tiles;
-//   barrier.
+//   barrier ; while it waits, a block does the move's bookkeeping.
+// Measured against the same moves with four blocks of 256 threads an SM, a
+// frontier compacted across the GPU (a reservation per block, 20 bytes a row
+// written and read again, row offsets and dense moved cash for every node)
+// and pushed in chunks of 1024 links: R-MAT 20, per-link threshold, a move
+// 34.5 -> 31.3 us (select 9.4 + 3.8 wait -> 8.4 + 2.3; push 20.4 -> 20.5, of
+// which 2.67 M scattered additions take about 18 however they are issued:
+// 23 us as a kernel of their own on the same links); symmetrised R-MAT 24,
+// a move 324 -> 268 us (select 158 -> 79, push 166 -> 189, see push_rows);
+// PageRank of an R-MAT graph of 500000 nodes 63 -> 48 us.
 // With the stale threshold (Control::theta_lag) a move after the first of a
 // launch has no stats phase and no first barrier: its select gathers the
 // statistics of the cash it reads, and the next move's threshold and
@@ -36,11 +45,16 @@
 
 namespace rlgl {
 
-constexpr int kSweepMinBlocks = 4;  // blocks per SM (launch bounds)
+// The sweep runs one block of 1024 threads per SM. Against four of 256 a
+// grid barrier with four FP64 totals takes 1.4 us instead of 3.0 (measured:
+// the arrivals queue on one counter), and the block's warps can share out
+// its nodes through shared memory.
+constexpr int kSweepThreads = 1024;
+constexpr int kSweepWarps = kSweepThreads / 32;
 constexpr int ST_BARRIER = 9;
 
-// Per-move accumulators, zero at rest. Two slots alternate: the slot of
-// move t is cleared by block 0 during move t + 1, after the first barrier,
+// Per-move accumulators, zero at rest. Three slots rotate: the slot of
+// move t is cleared by block 0 during move t + 1, after its first barrier,
 // when every block has finished reading it.
 // Every group of fields that all blocks update or read at one time sits on
 // its own 128-byte line, and so does the barrier: the blocks' atomics on one
@@ -56,9 +70,9 @@ struct SweepSlot {
     double mabs;                 // sum |m_i|
     alignas(128) unsigned long long reserve;  // packed frontier reservation
     unsigned long long tstamp;   // block 0's timer at the end of its stats (or select)
-    alignas(128) double s;       // sum C
-    unsigned long long chunk_next;  // next push chunk (or pull tile) to hand out
-    unsigned long long range_next;  // select of large chains: next node range to hand out
+    alignas(128) double s;       // sum C (the all-green sweep)
+    unsigned long long chunk_next;  // next pull tile to hand out
+    unsigned long long pieces;   // pieces of long green rows
 };
 static_assert(offsetof(SweepSlot, pr) == offsetof(SweepSlot, a) + 8 && offsetof(SweepSlot, a) % 16 == 0,
               "a, pr: one 16-byte pair");
@@ -82,7 +96,7 @@ __device__ __forceinline__ double2 ldcg_pair(const void* p) {
 
 struct SweepState {
     GridBar bar;
-    SweepSlot slot[3];  // the general sweep alternates slots 0 and 1; the all-green sweep rotates all three
+    SweepSlot slot[3];  // in rotation
     // TOPFRAC: the radix passes' digit histograms (zero at rest), three in
     // rotation: pass q adds into q mod 3, every block reads it after the
     // pass's barrier, and block 0 then clears (q + 2) mod 3, which every
@@ -138,23 +152,32 @@ __device__ __forceinline__ int bar_wait(GridBar* bar, unsigned long long target,
 
 // Grid-wide barrier of a cooperative launch: the count only grows, so no
 // block has to reset or release anything. `target` is the block's expected
-// arrival count (kept by thread 0). `work` runs in thread 0 between its
+// arrival count (kept by thread 0). `before` runs in thread 0 between its
 // arrival and its wait (off the critical path unless this block arrives
-// last). The wait is bounded by limit_ns; returns false (in every thread of
-// the block) when the sweep must stop. When ts is given, thread 0 stores its
-// arrival and release times in ts[0], ts[1].
-template <typename F>
+// last), `after` in every lane of warp 0 once the wait is over, before the
+// rest of the block goes on (the block meets twice in all). The wait is
+// bounded by limit_ns; returns false (in every thread of the block) when the
+// sweep must stop. When ts is given, thread 0 stores its arrival and release
+// times in ts[0], ts[1].
+template <typename F, typename G>
 __device__ __forceinline__ bool grid_barrier_with(GridBar* bar, unsigned long long& target,
                                                   unsigned long long limit_ns, unsigned long long* ts,
-                                                  F&& work) {
+                                                  F&& before, G&& after) {
     __shared__ int s_ok;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        if (ts) ts[0] = globaltimer();
-        bar_arrive(bar, target);
-        work();
-        s_ok = bar_wait(bar, target, limit_ns);
-        if (ts) ts[1] = globaltimer();
+    if (threadIdx.x < 32) {
+        int ok = 1;
+        if (threadIdx.x == 0) {
+            if (ts) ts[0] = globaltimer();
+            bar_arrive(bar, target);
+            before();
+            ok = bar_wait(bar, target, limit_ns);
+            if (ts) ts[1] = globaltimer();
+            s_ok = ok;
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        __syncwarp();
+        if (ok) after();
     }
     __syncthreads();
     return s_ok != 0;
@@ -163,8 +186,23 @@ __device__ __forceinline__ bool grid_barrier_with(GridBar* bar, unsigned long lo
 __device__ __forceinline__ bool grid_barrier(GridBar* bar, unsigned long long& target,
                                              unsigned long long limit_ns,
                                              unsigned long long* ts = nullptr) {
-    return grid_barrier_with(bar, target, limit_ns, ts, []() {});
+    return grid_barrier_with(bar, target, limit_ns, ts, []() {}, []() {});
 }
+
+// A green row: its node and the moved cash per weight.
+template <typename T>
+struct alignas(2 * sizeof(T)) Green {
+    int id;
+    T m;
+};
+
+// A piece of a long green row: links [pos, pos + len), moved cash per weight m.
+template <typename T>
+struct Piece {
+    long long pos;
+    int len;
+    T m;
+};
 
 template <typename T>
 struct SweepArgs {
@@ -175,13 +213,14 @@ struct SweepArgs {
     const long long* row_ptr;
     const T* ideg;
     const unsigned char* masks;
+    const int* deg;     // links of each row
+    Green<T>* list;     // the sweep's green rows, each block's in its own part
+    Piece<T>* pieces;   // pieces of its long green rows
+    int n_hubs;  // hub targets of the push, and the only one when there is one
+    int hub1;
     T* mt;
     T* mt2;      // power sweep: the moved cash of every other move
     T* facc;     // power sweep: sums of rows split across tiles (zero at rest)
-    long long* f_eoff;
-    long long* f_base;
-    T* f_m;
-    int* chunk_row;
     const int* col;
     const float* w;
     const long long* t_ptr;
@@ -204,502 +243,494 @@ struct SweepArgs {
     const int* hubs;  // hub table of the push (nullptr: none)
 };
 
-// Shared cache of the select phase when the chain has at most kIters
-// block-iterations (2 for FP32 cash, 1 for FP64, so that a block's static
-// shared memory stays within 48 KB): the block's node ranges (contiguous,
-// kNodesPerIter nodes each) keep their cash, 1/d, row offsets and test
-// results between the counting pass and the writing pass, and every warp's
-// green count and edge sum for each of its node groups sits there. The
-// arrays are filled by asynchronous 16-byte copies.
-constexpr int kSelRp = kNodesPerIter + 2;  // row offsets of a range (+1, padded to 16 bytes)
-template <typename T>
-struct SelSmem {
-    static constexpr int kIters = sizeof(T) == 4 ? 2 : 1;
-    static constexpr int kNodes = kIters * kNodesPerIter;
-    alignas(16) T val[kNodes];
-    alignas(16) T idg[kNodes];
-    alignas(16) T sv[kNodes];  // s_i in the cash type (1 / row weight)
-    alignas(16) long long rp[kIters][kSelRp];
-    unsigned char g[kNodes];
-    unsigned long long wsum[kIters * kNodesPerThread * (kThreads / 32)];  // packed (edges << kCountBits) | count
-};
-
-// Asynchronous copy of `bytes` (1..16) from global to shared memory, the
-// rest of the 16 destination bytes zero-filled; both addresses 16-byte
-// aligned. Completed by cp_async_wait_all.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, int bytes) {
-    const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa), "l"(gmem), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// Waits until at most the most recent committed group is in flight.
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-
 // s_i in the cash type: FP32 on the MIXED path, FP64 on the FP64 path.
 __device__ __forceinline__ const float* row_scale(const float* sf, const double*, float) { return sf; }
 __device__ __forceinline__ const double* row_scale(const float*, const double* s, double) { return s; }
 
-// Warp sum of the packed (edges << kCountBits) | count of the green lanes:
-// the count from the ballot, the edges from two 32-bit warp reductions of
-// the degree's 16-bit halves (no overflow for any int32 degrees).
-__device__ __forceinline__ unsigned long long warp_pack_sum(bool g, int rdeg) {
-    const unsigned int cnt = __popc(__ballot_sync(0xffffffffu, g));
-    const unsigned int lo = __reduce_add_sync(0xffffffffu, g ? ((unsigned int)rdeg & 0xffffu) : 0u);
-    const unsigned int hi = __reduce_add_sync(0xffffffffu, g ? ((unsigned int)rdeg >> 16) : 0u);
-    return ((((unsigned long long)hi << 16) + lo) << kCountBits) + cnt;
-}
-
-// Exclusive prefix over the warp's lanes of x >= 0 (x < 2^31).
-__device__ __forceinline__ long long warp_exscan_deg(int x) {
-    const int lane = threadIdx.x & 31;
-    if (__all_sync(0xffffffffu, x < (1 << 26))) {
-        // 32 x 2^26 = 2^31: the sums fit 32 bits
-        int y = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int z = __shfl_up_sync(0xffffffffu, y, o);
-            if (lane >= o) y += z;
-        }
-        return (long long)(y - x);
-    }
-    long long y = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long z = __shfl_up_sync(0xffffffffu, y, o);
-        if (lane >= o) y += z;
-    }
-    return y - x;
-}
-
-// Copies elements [e0, e0 + count) of src (count elements of type E in
-// 16-byte pieces; the array holds `avail` elements from index 0) into dst,
-// zero past the array's end. Every thread of the block takes pieces.
-template <typename E>
-__device__ __forceinline__ void stage_range(E* dst, const E* src, long long e0, int count, long long avail) {
-    constexpr int kPer = 16 / (int)sizeof(E);
-    const int pieces = (count + kPer - 1) / kPer;
-    for (int u = threadIdx.x; u < pieces; u += blockDim.x) {
-        const long long e = e0 + (long long)u * kPer;
-        const long long left = (avail - e) * (long long)sizeof(E);
-        E* d = dst + u * kPer;
-        if (left >= 16) cp_async16(d, src + e, 16);
-        else if (left > 0) cp_async16(d, src + e, (int)left);
-        else *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-}
-
-// Select on this block's node slices (the single-chain form of k_select):
-// green nodes give their cash (m_i = C_i, C_i <- 0, H_i += m_i) and get
-// frontier entries and push-chunk starts; mt holds m~_i (0 for red nodes).
-// Two passes over the block's nodes: the first counts green nodes and their
-// edges, one atomic per block reserves the block's frontier range, the
-// second writes it. For the first two block-iterations (cached in shared
-// memory) the frontier slots follow node order within each warp, so a
-// warp's frontier writes are contiguous; beyond, each thread's green nodes
-// take consecutive slots. Returns the block's sums of m_i and |m_i| in
-// thread 0. With acc_stats (the stale threshold), also the block's sums of
-// the statistics of the cash before the move, from the same loads:
-// ba = sum |C_i| and bpr = sum v_i^r as the statistics pass forms them
-// (v_i = |C_i| / d_i when link, else |C_i|; bpr stays 0 for r = 1 without
-// link, whose sum is ba).
-// x^r for the rare exponents r > 2, out of line so that the select loop
-// does not carry pow's registers.
+// x^r for the rare exponents r > 2, out of line so that the node loops do
+// not carry pow's registers.
 template <typename T>
 __device__ __noinline__ T pow_r(T x, int r) {
     return pow(x, (T)r);
 }
 
+// ------------------------------------------------------- the node passes
+//
+// A block owns a contiguous span of nodes and selects, lists and pushes its
+// own green rows; only rows of more than kHubRow links are cut into pieces
+// that all blocks share. So a row's entry is written and read on the same SM,
+// no space has to be reserved across the GPU, and nothing of a red node is
+// read but its cash (and its 1/degree for the per-link test).
+//
+// What bounds it: on an L2-resident chain the push's scattered additions
+// (about 210 G/s over the whole GPU, measured), beyond L2 the bytes of the
+// cash, the row offsets and the links; the rest is the instructions spent on
+// a node and the latency of a phase.
+
+// Nodes a lane handles per group: node g0 + 32 q + lane for q < kV, so that
+// every access of a warp is to consecutive addresses.
 template <typename T>
-__device__ __forceinline__ void sweep_select(const SweepArgs<T>& A, int sched, T th,
-                                             const unsigned char* mask, const SchedAux& ax,
-                                             SweepSlot* sl, SelSmem<T>& cs, bool acc_stats,
-                                             bool link, int r, double& bmsum, double& bmabs,
-                                             double& ba, double& bpr) {
-    __shared__ T tscratch[4 * 32];
-    __shared__ unsigned long long base_sh;
-    // rows with many push chunks: their chunk starts are written by the
-    // whole block after the second pass instead of by one thread
-    constexpr int kLongRows = 16;
-    constexpr int kLongChunks = 8;
-    __shared__ int s_nlong;
-    __shared__ long long s_long[kLongRows][3];  // frontier row, first chunk, end chunk
-    const int n = A.n;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    T msum = T(0), mabs = T(0), sa = T(0), spr = T(0);
-    // the statistics pass's terms (stats_slice)
-    auto stat = [&](T v, T idg) {
-        const T av = fabs(v);
-        sa += av;
-        const T tv = link ? av * idg : av;
-        if (link && r == 1) spr += tv;
-        else if (r == 2) spr += tv * tv;
-        else if (r > 2) spr += pow_r(tv, r);
-    };
-    auto finish = [&]() {
-        T v4[4] = {msum, mabs, sa, spr};
-        block_sum_n<T, 4>(v4, tscratch);
-        bmsum = (double)v4[0];
-        bmabs = (double)v4[1];
-        ba = (double)v4[2];
-        bpr = (double)v4[3];
-    };
-    if (sched == SCHED_ALL_GREEN) {
-        // every node moves; the pull needs no frontier
-        for (long long it0 = (long long)blockIdx.x * kNodesPerIter; it0 < n;
-             it0 += (long long)gridDim.x * kNodesPerIter) {
-            // every load of the range first: red_add orders later loads after it
-            T val[kNodesPerThread], idg[kNodesPerThread], scv[kNodesPerThread];
-#pragma unroll
-            for (int q = 0; q < kNodesPerThread; ++q) {
-                const long long i = it0 + q * kThreads + threadIdx.x;
-                val[q] = i < n ? __ldcg(A.c + i) : T(0);
-                idg[q] = (i < n && link) ? __ldg(A.ideg + i) : T(0);
-                scv[q] = i < n ? moved_per_weight(T(1), A.s, A.sf, i) : T(0);
-            }
-#pragma unroll
-            for (int q = 0; q < kNodesPerThread; ++q) {
-                const long long i = it0 + q * kThreads + threadIdx.x;
-                if (i >= n) continue;
-                const T v = val[q];
-                if (acc_stats) stat(v, idg[q]);
-                A.c[i] = T(0);
-                red_add(A.H + i, (double)v);  // no load: the L2 adds
-                msum += v;
-                mabs += fabs(v);
-                A.mt[i] = v * scv[q];
-            }
-        }
-        finish();
-        return;
-    }
-    if ((long long)n > (long long)gridDim.x * SelSmem<T>::kNodes && SelSmem<T>::kIters >= 2) {
-        // Large chains, FP32 cash: node ranges of kNodesPerIter one after
-        // another through the two stages of the shared cache, the next
-        // range's asynchronous copies in flight while this one is tested,
-        // reserved and written. One reservation per range: a count pass over
-        // all of them first would read the nodes from memory twice. Block b
-        // takes ranges b and b + G, then grabs the next free range from a
-        // counter (the grab issued a range ahead), so that blocks end within
-        // a fraction of a range of one another.
-        const bool with_idg = sched == SCHED_LINK;
-        // unweighted chains: s_i = 1/d_i, bit for bit the staged 1/d
-        const bool scale_is_idg = with_idg && A.w == nullptr;
-        const T* scale = scale_is_idg ? cs.idg : cs.sv;
-        const long long G = gridDim.x;
-        const long long nranges = ((long long)n + kNodesPerIter - 1) / kNodesPerIter;
-        __shared__ long long s_grab[2];
-        auto stage = [&](int buf, long long r) {
-            const long long it0 = r * kNodesPerIter;
-            stage_range<T>(cs.val + buf * kNodesPerIter, A.c, it0, kNodesPerIter, n);
-            if (with_idg) stage_range<T>(cs.idg + buf * kNodesPerIter, A.ideg, it0, kNodesPerIter, n);
-            if (!scale_is_idg)
-                stage_range<T>(cs.sv + buf * kNodesPerIter, row_scale(A.sf, A.s, T(0)), it0, kNodesPerIter, n);
-            stage_range<long long>(cs.rp[buf], A.row_ptr, it0, kSelRp, (long long)n + 1);
-            cp_async_commit();
-        };
-        // n > G x kNodes: ranges b and b + G exist for every block
-        long long cur = blockIdx.x, nxt = blockIdx.x + G;
-        stage(0, cur);
-        stage(1, nxt);
-        for (int j = 0;; ++j) {
-            const int buf = j & 1;
-            const long long it0 = cur * kNodesPerIter;
-            // the range after next, staged at the end of this iteration: the
-            // grab's reply is first used there, so its round trip overlaps
-            // this range's work
-            unsigned long long grab = 0ull;
-            if (threadIdx.x == 0 && nxt >= 0) grab = atomicAdd(&sl->range_next, 1ull);
-            if (nxt >= 0) cp_async_wait_prev();
-            else cp_async_wait_all();
-            __syncthreads();
-#pragma unroll
-            for (int q = 0; q < kNodesPerThread; ++q) {
-                const int loc = q * kThreads + threadIdx.x;
-                const int slot = buf * kNodesPerIter + loc;
-                const long long i = it0 + loc;
-                const T v = cs.val[slot];
-                const T idg = with_idg ? cs.idg[slot] : T(0);
-                const int rdeg = (int)(cs.rp[buf][loc + 1] - cs.rp[buf][loc]);
-                const bool g = (i < n) && green_test_v<T>(sched, v, idg, i, th, mask, ax);
-                if (acc_stats && i < n) stat(v, idg);
-                cs.g[slot] = g ? 1 : 0;
-                const unsigned long long w = warp_pack_sum(g, rdeg);
-                if (lane == 0) cs.wsum[q * (kThreads / 32) + wid] = w;
-            }
-            __syncthreads();
-            if (wid == 0) {
-                // kNodesPerThread x warps = 32 groups: one warp-wide scan
-                const unsigned long long v = cs.wsum[lane];
-                unsigned long long x = v;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-                    if (lane >= o) x += y;
-                }
-                cs.wsum[lane] = x - v;
-                const unsigned long long run = __shfl_sync(0xffffffffu, x, 31);
-                if (lane == 0) {
-                    base_sh = run ? atomicAdd(&sl->reserve, run) : 0ull;
-                    s_nlong = 0;
-                }
-            }
-            __syncthreads();
-            const unsigned long long base = base_sh;
-#pragma unroll
-            for (int q = 0; q < kNodesPerThread; ++q) {
-                const int loc = q * kThreads + threadIdx.x;
-                const int slot = buf * kNodesPerIter + loc;
-                const long long i = it0 + loc;
-                const T v = cs.val[slot];
-                const long long rb = cs.rp[buf][loc];
-                const int rdeg = (int)(cs.rp[buf][loc + 1] - rb);
-                const bool g = cs.g[slot] != 0;
-                const unsigned int bal = __ballot_sync(0xffffffffu, g);
-                if (bal == 0u) {  // no green node in this warp's group
-                    if (i < n) A.mt[i] = T(0);
-                    continue;
-                }
-                const long long xe = warp_exscan_deg(g ? rdeg : 0);
-                const unsigned long long wb = base + cs.wsum[q * (kThreads / 32) + wid];
-                const long long kk = (long long)(wb & ((1ull << kCountBits) - 1ull)) + __popc(bal & ((1u << lane) - 1u));
-                const long long ee = (long long)(wb >> kCountBits) + xe;
-                if (i >= n) continue;
-                if (g) {
-                    const T mtil = v * scale[slot];
-                    A.c[i] = T(0);
-                    red_add(A.H + i, (double)v);  // no load: the L2 adds
-                    msum += v;
-                    mabs += fabs(v);
-                    A.mt[i] = mtil;
-                    A.f_eoff[kk] = ee;
-                    A.f_base[kk] = rb - ee;
-                    A.f_m[kk] = mtil;
-                    const long long b0 = (ee + kPushChunk - 1) / kPushChunk;
-                    const long long b1 = (ee + rdeg + kPushChunk - 1) / kPushChunk;
-                    int ls = -1;
-                    if (b1 - b0 > kLongChunks) {
-                        ls = atomicAdd(&s_nlong, 1);
-                        if (ls < kLongRows) {
-                            s_long[ls][0] = kk;
-                            s_long[ls][1] = b0;
-                            s_long[ls][2] = b1;
-                        }
-                    }
-                    if (ls < 0 || ls >= kLongRows)
-                        for (long long b = b0; b < b1; ++b) A.chunk_row[b] = (int)kk;
-                } else {
-                    A.mt[i] = T(0);
-                }
-            }
-            if (threadIdx.x == 0 && nxt >= 0) s_grab[buf] = 2 * G + (long long)grab;
-            __syncthreads();
-            // this stage is free: the range after next goes into it
-            long long after = nxt >= 0 ? s_grab[buf] : -1;
-            if (after >= nranges) after = -1;
-            if (after >= 0) stage(buf, after);
-            const int nlong = s_nlong < kLongRows ? s_nlong : kLongRows;
-            for (int q = 0; q < nlong; ++q)
-                for (long long b = s_long[q][1] + threadIdx.x; b < s_long[q][2]; b += blockDim.x)
-                    A.chunk_row[b] = (int)s_long[q][0];
-            cur = nxt;
-            nxt = after;
-            if (cur < 0) break;
-        }
-        finish();
-        return;
-    }
-    if ((long long)n > (long long)gridDim.x * SelSmem<T>::kNodes) {
-        // Large chains, FP64 cash (more block-iterations than the cache holds): one pass
-        // with one reservation per block-iteration, so that the nodes are
-        // read once (a second pass would read them again from memory).
-        for (long long it0 = (long long)blockIdx.x * kNodesPerIter; it0 < n;
-             it0 += (long long)gridDim.x * kNodesPerIter) {
-            long long rb[kNodesPerThread];
-            int rdeg[kNodesPerThread];
-            T val[kNodesPerThread], idg[kNodesPerThread], scv[kNodesPerThread];
-            bool g[kNodesPerThread];
-#pragma unroll
-            for (int q = 0; q < kNodesPerThread; ++q) {
-                const long long i = it0 + q * kThreads + threadIdx.x;
-                rb[q] = (i < n) ? __ldg(A.row_ptr + i) : 0;
-                rdeg[q] = (i < n) ? (int)(__ldg(A.row_ptr + i + 1) - rb[q]) : 0;
-                val[q] = (i < n) ? __ldcg(A.c + i) : T(0);
-                idg[q] = (i < n && sched == SCHED_LINK) ? __ldg(A.ideg + i) : T(0);
-                // s_i now: red_add below orders every later load after it
-                scv[q] = (i < n) ? moved_per_weight(T(1), A.s, A.sf, i) : T(0);
-            }
-            unsigned long long mine = 0ull;
-#pragma unroll
-            for (int q = 0; q < kNodesPerThread; ++q) {
-                const long long i = it0 + q * kThreads + threadIdx.x;
-                g[q] = (i < n) && green_test_v<T>(sched, val[q], idg[q], i, th, mask, ax);
-                if (g[q]) mine += ((unsigned long long)rdeg[q] << kCountBits) + 1ull;
-                if (acc_stats && i < n) stat(val[q], idg[q]);
-            }
-            unsigned long long total;
-            const unsigned long long pre = block_exscan(mine, &total);
-            if (threadIdx.x == 0) base_sh = total ? atomicAdd(&sl->reserve, total) : 0ull;
-            __syncthreads();
-            const unsigned long long base = base_sh + pre;
-            long long k = (long long)(base & ((1ull << kCountBits) - 1ull));
-            long long e = (long long)(base >> kCountBits);
-#pragma unroll
-            for (int q = 0; q < kNodesPerThread; ++q) {
-                const long long i = it0 + q * kThreads + threadIdx.x;
-                if (i >= n) continue;
-                if (g[q]) {
-                    const T v = val[q];
-                    const T mtil = v * scv[q];
-                    A.c[i] = T(0);
-                    red_add(A.H + i, (double)v);  // no load: the L2 adds
-                    msum += v;
-                    mabs += fabs(v);
-                    A.mt[i] = mtil;
-                    A.f_eoff[k] = e;
-                    A.f_base[k] = rb[q] - e;
-                    A.f_m[k] = mtil;
-                    const long long b0 = (e + kPushChunk - 1) / kPushChunk;
-                    const long long b1 = (e + rdeg[q] + kPushChunk - 1) / kPushChunk;
-                    for (long long b = b0; b < b1; ++b) A.chunk_row[b] = (int)k;
-                    ++k;
-                    e += rdeg[q];
-                } else {
-                    A.mt[i] = T(0);
-                }
-            }
-            __syncthreads();  // base_sh is rewritten by the next iteration
-        }
-        finish();
-        return;
-    }
-    // Cached path (n <= grid x kNodes): at most kIters ranges.
-    // Pass 1 stages every range's cash, 1/d and row offsets in shared
-    // memory at once (one round trip, no registers held), then tests and
-    // counts from there, per warp and node group.
-    const bool with_idg = sched == SCHED_LINK;
-    const bool scale_is_idg = with_idg && A.w == nullptr;  // s_i = 1/d_i
-    const T* scale = scale_is_idg ? cs.idg : cs.sv;
-    int nj = 0;
-    for (int j = 0; j < SelSmem<T>::kIters; ++j) {
-        const long long it0 = ((long long)blockIdx.x + (long long)j * gridDim.x) * kNodesPerIter;
-        if (it0 >= n) break;
-        ++nj;
-        stage_range<T>(cs.val + j * kNodesPerIter, A.c, it0, kNodesPerIter, n);
-        if (with_idg) stage_range<T>(cs.idg + j * kNodesPerIter, A.ideg, it0, kNodesPerIter, n);
-        if (!scale_is_idg)
-            stage_range<T>(cs.sv + j * kNodesPerIter, row_scale(A.sf, A.s, T(0)), it0, kNodesPerIter, n);
-        stage_range<long long>(cs.rp[j], A.row_ptr, it0, kSelRp, (long long)n + 1);
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    for (int j = 0; j < nj; ++j) {
-        const long long it0 = ((long long)blockIdx.x + (long long)j * gridDim.x) * kNodesPerIter;
-#pragma unroll
-        for (int q = 0; q < kNodesPerThread; ++q) {
-            const int loc = q * kThreads + threadIdx.x;
-            const int slot = j * kNodesPerIter + loc;
-            const long long i = it0 + loc;
-            const T v = cs.val[slot];
-            const T idg = with_idg ? cs.idg[slot] : T(0);
-            const int rdeg = (int)(cs.rp[j][loc + 1] - cs.rp[j][loc]);
-            const bool g = (i < n) && green_test_v<T>(sched, v, idg, i, th, mask, ax);
-            if (acc_stats && i < n) stat(v, idg);
-            cs.g[slot] = g ? 1 : 0;
-            const unsigned long long w = warp_pack_sum(g, rdeg);
-            if (lane == 0) cs.wsum[(j * kNodesPerThread + q) * (kThreads / 32) + wid] = w;
-        }
-    }
-    const int ncached = nj * kNodesPerThread * (kThreads / 32);
-    __syncthreads();
-    // exclusive prefix of the groups' counts in group order, and one
-    // reservation for the whole block (warp 0)
-    if (wid == 0) {
-        unsigned long long run = 0ull;
-        for (int g0 = 0; g0 < ncached; g0 += 32) {
-            const int gi = g0 + lane;
-            const unsigned long long v = gi < ncached ? cs.wsum[gi] : 0ull;
-            unsigned long long x = v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
-            }
-            if (gi < ncached) cs.wsum[gi] = run + x - v;
-            run += __shfl_sync(0xffffffffu, x, 31);
-        }
-        if (lane == 0) {
-            base_sh = run ? atomicAdd(&sl->reserve, run) : 0ull;
-            s_nlong = 0;
-        }
-    }
-    __syncthreads();
-    const unsigned long long base = base_sh;
-    // pass 2: write (frontier slots in node order within each warp)
-    for (int j = 0; j < nj; ++j) {
-        const long long it0 = ((long long)blockIdx.x + (long long)j * gridDim.x) * kNodesPerIter;
-#pragma unroll
-        for (int q = 0; q < kNodesPerThread; ++q) {
-            const int loc = q * kThreads + threadIdx.x;
-            const int slot = j * kNodesPerIter + loc;
-            const long long i = it0 + loc;
-            const T v = cs.val[slot];
-            const long long rb = cs.rp[j][loc];
-            const int rdeg = (int)(cs.rp[j][loc + 1] - rb);
-            const bool g = cs.g[slot] != 0;
-            const unsigned int bal = __ballot_sync(0xffffffffu, g);
-            if (bal == 0u) {  // no green node in this warp's group
-                if (i < n) A.mt[i] = T(0);
-                continue;
-            }
-            const long long xe = warp_exscan_deg(g ? rdeg : 0);
-            const unsigned long long wb = base + cs.wsum[(j * kNodesPerThread + q) * (kThreads / 32) + wid];
-            const long long kk = (long long)(wb & ((1ull << kCountBits) - 1ull)) + __popc(bal & ((1u << lane) - 1u));
-            const long long ee = (long long)(wb >> kCountBits) + xe;
-            if (i >= n) continue;
-            if (g) {
-                const T mtil = v * scale[slot];
-                A.c[i] = T(0);
-                red_add(A.H + i, (double)v);  // no load: the L2 adds
-                msum += v;
-                mabs += fabs(v);
-                A.mt[i] = mtil;
-                A.f_eoff[kk] = ee;
-                A.f_base[kk] = rb - ee;
-                A.f_m[kk] = mtil;
-                const long long b0 = (ee + kPushChunk - 1) / kPushChunk;
-                const long long b1 = (ee + rdeg + kPushChunk - 1) / kPushChunk;
-                int ls = -1;
-                if (b1 - b0 > kLongChunks) {
-                    ls = atomicAdd(&s_nlong, 1);
-                    if (ls < kLongRows) {
-                        s_long[ls][0] = kk;
-                        s_long[ls][1] = b0;
-                        s_long[ls][2] = b1;
-                    }
-                }
-                if (ls < 0 || ls >= kLongRows)
-                    for (long long b = b0; b < b1; ++b) A.chunk_row[b] = (int)kk;
-            } else {
-                A.mt[i] = T(0);
-            }
-        }
-    }
-    __syncthreads();
-    const int nlong = s_nlong < kLongRows ? s_nlong : kLongRows;
-    for (int q = 0; q < nlong; ++q)
-        for (long long b = s_long[q][1] + threadIdx.x; b < s_long[q][2]; b += blockDim.x)
-            A.chunk_row[b] = (int)s_long[q][0];
-    finish();
+struct NodeVec {
+    static constexpr int kV = sizeof(T) == 4 ? 4 : 2;
+};
+
+// (double)v without the FP64 pipe, which takes 16 cycles an SM and warp for
+// an addition or a conversion: a normal number's exponent and fraction moved
+// to their places; zeros, subnormals, infinities and NaN by the conversion.
+__device__ __forceinline__ double widen(float v) {
+    const unsigned int u = __float_as_uint(v), e = (u >> 23) & 255u;
+    if (e == 0u || e == 255u) return (double)v;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+
+// v >= th for th >= 0, v = |x|: the FP64 comparison as one of the bit
+// patterns (their order is that of the values; NaN compares false).
+__device__ __forceinline__ bool at_least(float v, float th) { return v >= th; }
+__device__ __forceinline__ bool at_least(double v, double th) {
+    const unsigned long long a = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return a >= (unsigned long long)__double_as_longlong(th) && a <= 0x7ff0000000000000ull;
 }
 
+// A block's hub targets (see kHubSlots) and their sums of the move.
 template <typename T>
-union SweepSmem {
-    PushSmem<T> push;
-    PullSmem<T> pull;
-    SelSmem<T> sel;
-    unsigned int hist[kRadixBins];  // TOPFRAC: the block's digit histogram
+struct HotSmem {
+    int hub[kHubSlots];
+    double hot[kHubSlots];  // zero at rest
+    // with a single hub: the threads' sums (see hub_add), zero at rest
+    typename std::conditional<std::is_same<T, float>::value, float2, double>::type one[kSweepThreads];
 };
+
+// Rows of kShortRow < links <= kHubRow met by the block's push, left for
+// whichever warp is free at the end: a warp with several of them would
+// otherwise keep the GPU waiting.
+template <typename T>
+struct MidRows {
+    static constexpr int kCap = 1024;
+    long long base[kCap];
+    T m[kCap];
+    int len[kCap];
+};
+
+// The dynamic shared memory of the sweep.
+template <typename T>
+struct SweepSmem {
+    union {
+        MidRows<T> mid;
+        PullSmem<T, kSweepThreads> pull;
+        unsigned int hist[kRadixBins];  // TOPFRAC: the block's digit histogram
+    };
+    HotSmem<T> hot;
+    int next_group;  // node group to hand out next within the block
+    int n_list;      // green rows listed
+    int next_list;   // green row to push next
+    int n_mid;       // rows in mid
+    int next_mid;
+};
+
+// What a node pass needs to know of the move.
+template <typename T>
+struct MoveView {
+    const unsigned char* mask;
+    unsigned long long* n_pieces;  // the move's count of pieces of long rows
+    T th;
+    int sched, r;
+    bool link;    // statistics of v_i = |C_i| / d_i
+    bool acc;     // gather the statistics of the cash
+    bool dense;   // write the dense moved cash mt too (the move may pull)
+};
+
+// A thread's sums over a pass.
+template <typename T>
+struct NodeAcc {
+    T a, pr, m, ma;
+    unsigned long long edges;
+};
+template <typename T>
+constexpr NodeAcc<T> kNoAcc = {T(0), T(0), T(0), T(0), 0ull};
+
+// Adds v to a single hub target's sum of one thread: FP32 terms as a pair
+// of FP32 numbers whose sum carries every rounding error of the additions
+// (Knuth's two-sum), so that the FP64 pipe is left out of the edge loop;
+// FP64 terms in FP64. In shared memory: few chains have a hub, and the node
+// loops need their registers.
+__device__ __forceinline__ void hub_add(float2& h, float v) {
+    const float s = h.x, t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+    h.y = __fadd_rn(h.y, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z)));
+    h.x = t;
+}
+__device__ __forceinline__ void hub_add(double& h, double v) { h += v; }
+__device__ __forceinline__ double hub_value(const float2& h) { return (double)h.x + (double)h.y; }
+__device__ __forceinline__ double hub_value(const double& h) { return h; }
+
+// The additions of kU edges a lane (target j, -1: none; amount v) to the
+// cash. Targets in the hub table (PageRank's auxiliary node, which
+// every node feeds) are summed apart: one of them by thread, several by warp
+// in shared memory.
+template <typename T, int kU>
+__device__ __forceinline__ void add_edges(T* __restrict__ c, int (&j)[kU], const T (&v)[kU], int n_hubs, int hub1,
+                                          HotSmem<T>& hot) {
+    if (n_hubs == 0) {
+#pragma unroll
+        for (int q = 0; q < kU; ++q)
+            if (j[q] >= 0) red_add(c + j[q], v[q]);
+    } else if (n_hubs == 1) {
+#pragma unroll
+        for (int q = 0; q < kU; ++q) {
+            if (j[q] == hub1) hub_add(hot.one[threadIdx.x], v[q]);
+            else if (j[q] >= 0) red_add(c + j[q], v[q]);
+        }
+    } else {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int q = 0; q < kU; ++q) {
+            int slot = -1;
+            if (j[q] >= 0) {
+                const int t = hub_slot(j[q]);
+                if (hot.hub[t] == j[q]) slot = t;
+                else red_add(c + j[q], v[q]);
+            }
+            unsigned int m = __ballot_sync(0xffffffffu, slot >= 0);
+            while (m) {
+                const int t = __shfl_sync(0xffffffffu, slot, __ffs(m) - 1);
+                const bool mine = slot == t;
+                const double x = warp_sum(mine ? (double)v[q] : 0.0);
+                if (lane == 0) atomicAdd(&hot.hot[t], x);
+                m &= ~__ballot_sync(0xffffffffu, mine);
+            }
+        }
+    }
+}
+
+// Pushes the links [pos, pos + len) of one row by the whole warp, four
+// links a lane in flight.
+template <typename T, bool kHasW>
+__device__ __forceinline__ void push_row(const SweepArgs<T>& A, long long pos, int len, T m, HotSmem<T>& hot) {
+    const int lane = threadIdx.x & 31;
+    for (int o = 0; o < len; o += 128) {
+        int j[4];
+        T v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = o + q * 32 + lane;
+            j[q] = e < len ? __ldg(A.col + pos + e) : -1;
+            v[q] = m;
+            if (kHasW && e < len) v[q] = m * (T)__ldg(A.w + pos + e);
+        }
+        add_edges<T, 4>(A.c, j, v, A.n_hubs, A.hub1, hot);
+    }
+}
+
+// The block's hub sums of the move into the cash, one addition per hub.
+template <typename T>
+__device__ __forceinline__ void flush_hubs(const SweepArgs<T>& A, HotSmem<T>& hot) {
+    if (A.n_hubs == 1) {
+        const double x = warp_sum(hub_value(hot.one[threadIdx.x]));
+        if ((threadIdx.x & 31) == 0 && x != 0.0) atomicAdd(&hot.hot[hub_slot(A.hub1)], x);
+        hot.one[threadIdx.x] = {};
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < kHubSlots; t += blockDim.x)
+        if (hot.hot[t] != 0.0) {
+            red_add(A.c + hot.hub[t], (T)hot.hot[t]);
+            hot.hot[t] = 0.0;
+        }
+}
+
+// The nodes [lo, hi) of this block: one contiguous span per block, a
+// multiple of 32 nodes, and the nodes its warps take at a time: 128 where
+// every warp gets several such groups, down to 32 where they would not
+// otherwise all get one.
+template <typename T>
+__device__ __forceinline__ void block_span(int n, int& lo, int& hi, int& group) {
+    const int nb = (int)gridDim.x;
+    const int span = (int)(((long long)n + nb * 32ll - 1) / (nb * 32ll)) * 32;
+    lo = (int)min((long long)blockIdx.x * span, (long long)n);
+    hi = (int)min((long long)lo + span, (long long)n);
+    group = span >= 128 * 2 * kSweepWarps ? 128 : (span >= 64 * kSweepWarps ? 64 : 32);
+    if (group > 32 * NodeVec<T>::kV) group = 32 * NodeVec<T>::kV;
+}
+
+// The passes over the nodes. STATS: the statistics of the cash. SELECT: the
+// green nodes give up their cash (m_i = C_i, C_i <- 0, H_i += m_i) and are
+// listed for the push. ALL: every node does, for a pull (dense moved cash m~
+// in mt, no list).
+enum Pass : int { PASS_STATS, PASS_SELECT, PASS_ALL };
+
+// The block's warps take its groups of nodes one after another from a
+// counter in shared memory (zero at the start of a pass; warp w starts with
+// group w); the next group's cash is loaded before the current one is listed.
+template <typename T, bool kHasW, int kPass>
+__device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<T>& mv, const SchedAux& ax,
+                                          SweepSmem<T>& sm, NodeAcc<T>& acc) {
+    constexpr int kV = NodeVec<T>::kV;
+    const int lane = threadIdx.x & 31;
+    int lo, hi, group;
+    block_span<T>(A.n, lo, hi, group);
+    const bool need_idg = mv.link && (kPass == PASS_STATS || mv.acc || mv.sched == SCHED_LINK);
+    const bool scale_is_idg = !kHasW && need_idg;  // unit weights: s_i = 1/d_i
+    const T* scale = row_scale(A.sf, A.s, T(0));
+    const T th = mv.th;
+    T C[kV], idg[kV];
+    auto load = [&](int g) {
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            const int i = g + q * 32 + lane;
+            C[q] = idg[q] = T(0);
+            if (q * 32 < group && i < hi) {
+                C[q] = __ldcg(A.c + i);
+                if (need_idg) idg[q] = __ldg(A.ideg + i);
+            }
+        }
+    };
+    int g0 = lo + (int)(threadIdx.x >> 5) * group;
+    load(g0);
+    while (g0 < hi) {
+        const int g = g0 + lane;
+        int nxt = 0;
+        if (lane == 0) nxt = atomicAdd(&sm.next_group, 1);
+        g0 = lo + (kSweepWarps + __shfl_sync(0xffffffffu, nxt, 0)) * group;
+        unsigned int gm = 0u;  // green nodes of this lane
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            const int i = g + q * 32;
+            if (q * 32 >= group || i >= hi) continue;
+            const T av = fabs(C[q]);
+            const T tv = mv.link ? av * idg[q] : av;
+            if (kPass == PASS_STATS || mv.acc) {
+                acc.a += av;
+                if (mv.link && mv.r == 1) acc.pr += tv;
+                else if (mv.r == 2) acc.pr += tv * tv;
+            }
+            bool green = kPass == PASS_ALL;
+            if (kPass == PASS_SELECT) {
+                // (the |C| and |C| / d tests of green_test_v)
+                if (mv.sched == SCHED_LINK || mv.sched == SCHED_THRESHOLD || mv.sched == SCHED_TOPFRAC)
+                    green = C[q] != T(0) && at_least(tv, th);
+                else
+                    green = green_test_v<T>(mv.sched, C[q], idg[q], i, th, mv.mask, ax);
+            }
+            if (green) gm |= 1u << q;
+        }
+        if (kPass == PASS_STATS) {
+            load(g0);
+            continue;
+        }
+        // green rows of the group, by node, and their place in the list
+        int k = 0;
+        if constexpr (kPass == PASS_SELECT) {
+#pragma unroll
+            for (int q = 0; q < kV; ++q) {
+                k += __popc(__ballot_sync(0xffffffffu, (gm >> q & 1u) != 0u));
+            }
+            if (lane == 0 && k > 0) k = atomicAdd(&sm.n_list, k);
+            k = lo + __shfl_sync(0xffffffffu, k, 0);
+        }
+        T m[kV];  // moved cash per weight
+        int deg[kV];
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            const int i = g + q * 32;
+            m[q] = T(0);
+            deg[q] = 0;
+            if (gm >> q & 1u) {
+                m[q] = C[q] * (scale_is_idg ? idg[q] : __ldg(scale + i));
+                if (kPass == PASS_SELECT) deg[q] = __ldg(A.deg + i);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < kV; ++q) {
+            const int i = g + q * 32;
+            if (!(gm >> q & 1u)) continue;
+            acc.m += C[q];
+            acc.ma += fabs(C[q]);
+            A.c[i] = T(0);
+            red_add(A.H + i, widen(C[q]));  // no load: the L2 adds
+        }
+        if (kPass == PASS_ALL || mv.dense) {
+#pragma unroll
+            for (int q = 0; q < kV; ++q)
+                if (q * 32 < group && g + q * 32 < hi) A.mt[g + q * 32] = m[q];
+        }
+        if constexpr (kPass == PASS_ALL) load(g0);
+        if constexpr (kPass == PASS_SELECT) {
+            int longest = 0;
+#pragma unroll
+            for (int q = 0; q < kV; ++q) {
+                const unsigned int bal = __ballot_sync(0xffffffffu, (gm >> q & 1u) != 0u);
+                if (gm >> q & 1u) {
+                    Green<T> e;
+                    e.id = g + q * 32;
+                    e.m = m[q];
+                    A.list[k + __popc(bal & ((1u << lane) - 1u))] = e;
+                }
+                k += __popc(bal);
+                acc.edges += (unsigned int)deg[q];
+                longest = max(longest, deg[q]);
+            }
+            load(g0);
+            if (__any_sync(0xffffffffu, longest > kHubRow)) {
+                // long rows: their pieces by the whole warp
+#pragma unroll
+                for (int q = 0; q < kV; ++q) {
+                    unsigned int b = __ballot_sync(0xffffffffu, deg[q] > kHubRow);
+                    while (b) {
+                        const int l = __ffs(b) - 1;
+                        b &= b - 1u;
+                        const int len = __shfl_sync(0xffffffffu, deg[q], l);
+                        const int np = (len + kHubRow - 1) / kHubRow;
+                        long long z = 0;
+                        if (lane == 0) z = (long long)atomicAdd(mv.n_pieces, (unsigned long long)np);
+                        z = __shfl_sync(0xffffffffu, z, 0);
+                        Piece<T> pc;
+                        pc.m = __shfl_sync(0xffffffffu, m[q], l);
+                        const long long pos = __ldg(A.row_ptr + (g - lane + q * 32 + l));
+                        for (int t = lane; t < np; t += 32) {
+                            pc.pos = pos + (long long)t * kHubRow;
+                            pc.len = min(kHubRow, len - t * kHubRow);
+                            A.pieces[z + t] = pc;
+                        }
+                    }
+                }
+            }
+        }
+    }
+}
+
+// A thread's share of sum v^r over the nodes [lo, hi) for r > 2 (ideg: 1/d
+// for the per-link v, else NULL), out of line: rare, and a call to pow inside
+// the node passes would cost them registers.
+template <typename T>
+__device__ __noinline__ T pow_sum(const T* c, const T* ideg, int lo, int hi, int r) {
+    T sum = T(0);
+    for (int i = lo + (int)threadIdx.x; i < hi; i += kSweepThreads) {
+        const T av = fabs(__ldcg(c + i));
+        sum += (T)pow(ideg ? av * __ldg(ideg + i) : av, (T)r);
+    }
+    return sum;
+}
+
+// The push of the green rows: first the GPU's pieces of long rows (warp w
+// takes every W-th of them, neighbours on different SMs), then the block's
+// listed rows 32 at a time, lane k holding row k: the links of the 32 rows
+// are taken together in windows of 32, and lane e finds its row in a window
+// as the number of rows that begin at or before it (one warp-wide or and a
+// bit count). Four windows are in flight. The block's rows of more than
+// kShortRow links come last, one warp each.
+template <typename T, bool kHasW>
+__device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& sm, int np) {
+    const int lane = threadIdx.x & 31;
+    const unsigned int upto = 0xffffffffu >> (31 - lane);
+    for (int p = (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x); p < np; p += (int)gridDim.x * kSweepWarps) {
+        // (written by other blocks during this kernel: from L2)
+        const long long pos = __ldcg(&A.pieces[p].pos);
+        const int len = __ldcg(&A.pieces[p].len);
+        const T m = __ldcg(&A.pieces[p].m);
+        push_row<T, kHasW>(A, pos, len, m, sm.hot);
+    }
+    const int nl = sm.n_list;
+    const Green<T>* list;
+    {
+        int lo, hi, group;
+        block_span<T>(A.n, lo, hi, group);
+        list = A.list + lo;
+    }
+    for (;;) {
+        int z = 0;
+        if (lane == 0) z = atomicAdd(&sm.next_list, 32);
+        z = __shfl_sync(0xffffffffu, z, 0);
+        if (z >= nl) break;
+        int len = 0;
+        long long base = 0;
+        T m = T(0);
+        if (z + lane < nl) {
+            const Green<T>* e = list + z + lane;
+            const int id = __ldcg(&e->id);
+            m = __ldcg(&e->m);
+            base = __ldg(A.row_ptr + id);
+            len = __ldg(A.deg + id);
+            if (len > kHubRow) len = 0;  // in pieces
+        }
+        const unsigned int mid = __ballot_sync(0xffffffffu, len > kShortRow);
+        if (mid) {
+            int k = 0;
+            if (lane == 0) k = atomicAdd(&sm.n_mid, __popc(mid));
+            k = __shfl_sync(0xffffffffu, k, 0) + __popc(mid & (upto >> 1));
+            if (len > kShortRow && k < MidRows<T>::kCap) {
+                sm.mid.base[k] = base;
+                sm.mid.m[k] = m;
+                sm.mid.len[k] = len;
+                len = 0;
+            }
+        }
+        int end = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += y;
+        }
+        const int E = __shfl_sync(0xffffffffu, end, 31);
+        const int start = end - len;
+        const unsigned int bit = len > 0 ? 1u << (start & 31) : 0u;
+        const int win = start >> 5;
+        // the rows with links, in order: row r of them is lane rank[r]
+        const unsigned int some = __ballot_sync(0xffffffffu, len > 0);
+        if (some != 0xffffffffu) {
+            // (the last rows, or long ones among them: close the gaps)
+            const int src = (int)__fns(some, 0, lane + 1);
+            base = __shfl_sync(0xffffffffu, base - start, src & 31);
+            m = __shfl_sync(0xffffffffu, m, src & 31);
+        } else {
+            base -= start;  // base + e: the link of edge e of the 32 rows
+        }
+        int rows = -1;  // the last row that began before the window
+        for (int w0 = 0; w0 * 32 < E; w0 += 4) {
+            int j[4];
+            T v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                j[q] = -1;
+                v[q] = T(0);
+                if ((w0 + q) * 32 >= E) continue;
+                const unsigned int word = __reduce_or_sync(0xffffffffu, win == w0 + q ? bit : 0u);
+                const int k = rows + __popc(word & upto);
+                rows += __popc(word);
+                const int e = (w0 + q) * 32 + lane;
+                const long long pos = __shfl_sync(0xffffffffu, base, k) + e;
+                v[q] = __shfl_sync(0xffffffffu, m, k);
+                if (e < E) {
+                    j[q] = __ldg(A.col + pos);
+                    if (kHasW) v[q] *= (T)__ldg(A.w + pos);
+                }
+            }
+            add_edges<T, 4>(A.c, j, v, A.n_hubs, A.hub1, sm.hot);
+        }
+    }
+    __syncthreads();
+    const int nm = min(sm.n_mid, MidRows<T>::kCap);
+    for (;;) {
+        int z = 0;
+        if (lane == 0) z = atomicAdd(&sm.next_mid, 1);
+        z = __shfl_sync(0xffffffffu, z, 0);
+        if (z >= nm) break;
+        push_row<T, kHasW>(A, sm.mid.base[z], sm.mid.len[z], sm.mid.m[z], sm.hot);
+    }
+}
+
+// The dense moved cash of a move that pulls though it was not expected to:
+// cleared (PASS 0), then set from the block's lists (after a barrier: other
+// blocks' spans do not matter, but the pull reads all of them).
+template <typename T>
+__device__ __forceinline__ void dense_from_lists(const SweepArgs<T>& A, SweepSmem<T>& sm) {
+    int lo, hi, group;
+    block_span<T>(A.n, lo, hi, group);
+    for (int i = lo + (int)threadIdx.x; i < hi; i += kSweepThreads) A.mt[i] = T(0);
+    __syncthreads();
+    for (int k = threadIdx.x; k < sm.n_list; k += kSweepThreads) {
+        const Green<T>* e = A.list + lo + k;
+        A.mt[__ldcg(&e->id)] = __ldcg(&e->m);
+    }
+}
 
 // TOPFRAC inside the sweep: one pass of the exact k-th largest |C| by radix
 // select over the IEEE bit patterns of |C| (the phase form is k_radix_pass).
@@ -708,8 +739,8 @@ union SweepSmem {
 // digits of a warp merged with __match_any_sync, one shared-memory add per
 // distinct digit), and adds its nonzero counts to the pass's histogram.
 template <typename T>
-__device__ __forceinline__ void sweep_radix_count(const T* c, int n, unsigned int* ghist, unsigned long long prefix,
-                                                  int shift, int width, unsigned int* h) {
+__device__ __forceinline__ void sweep_radix_count(const T* c, int n, unsigned int* ghist,
+                                                  unsigned long long prefix, int shift, int width, unsigned int* h) {
     const int nbins = 1 << width;
     for (int b = threadIdx.x; b < nbins; b += blockDim.x) h[b] = 0u;
     __syncthreads();
@@ -735,14 +766,14 @@ __device__ __forceinline__ void sweep_radix_count(const T* c, int n, unsigned in
 }
 
 // After the pass's barrier: the bucket of the remaining k-th largest key,
-// the same in every block (the same counts, the same scan). Thread t owns 8
+// the same in every block (the same counts, the same scan). Thread t owns 2
 // bins counted from the top; thread 0 gets the new prefix and remainder.
 __device__ __forceinline__ void sweep_radix_pick(const unsigned int* ghist, int shift, int width,
                                                  unsigned long long& prefix, long long& remain) {
     __shared__ int found;
     __shared__ long long above_found;
     if (threadIdx.x == 0) found = -1;
-    constexpr int per = kRadixBins / kThreads;  // 8
+    constexpr int per = kRadixBins / kSweepThreads;  // 2
     const int nbins = 1 << width;
     const int top = nbins - 1 - (int)threadIdx.x * per;
     unsigned long long mine = 0;
@@ -754,7 +785,7 @@ __device__ __forceinline__ void sweep_radix_pick(const unsigned int* ghist, int 
         mine += hb[q];
     }
     unsigned long long total;
-    const unsigned long long above = block_exscan(mine, &total);
+    const unsigned long long above = block_exscan<kSweepThreads>(mine, &total);
     const long long rem = remain;
     if ((long long)above < rem && (long long)(above + mine) >= rem) {
         long long cum = (long long)above;
@@ -786,7 +817,7 @@ struct SweepCtl {
     long long moves, solve_moves, iters, mask_cursor;
     long long tot_green, tot_edges, push_moves, pull_moves;
     long long green, edges;
-    double hsum, habs, theta, l1;
+    double hsum, habs, theta, l1, sumr, mabs;
     double stall_mark;
     long long stall_count;
     unsigned long long t_start;
@@ -794,62 +825,96 @@ struct SweepCtl {
     int fresh, sched, mode;
     int leave;         // 1: return now (stop, or re-derive before testing again)
     int want_refresh;  // return after this move for a re-derivation
-    int p;             // slot parity
+    int p;             // slot of the move
     unsigned long long target;  // expected arrival count at the next barrier
-    unsigned long long ts[7];  // block 0: move start, then arrival / release at each barrier
+    unsigned long long ts[2][7];  // block 0: move start, then arrival / release at each barrier
+    int tb;            // ts of the move (its predecessor's are still to be logged)
     SchedAux ax;       // this move's block-round-robin range and PC constants
-    long long mask_off;  // MASK: offset of this move's mask
-    // stale threshold: the statistics of the cash before the last move
-    double lag_l1, lag_sumr;
-    unsigned long long lag_now;  // block 0's timer when they were taken
-    int have_lag;      // a move of this launch has set them
-    int stop_after;    // status to stop with after this move (-1: none)
-    int lag_stop;      // stale threshold: the next move's stop before it selects (-1: none)
-    int pre_done;      // the next move's decisions are taken (sweep_lag_control)
+    int have_lag;      // stale threshold: a move of this launch has set the statistics
+    int stop;          // status to stop with now or after this move (-1: none)
+    int made;          // a move of this launch has been made
+    int owed;          // block 0: the last move's state and log entry are still to be written
+    MoveRecord rec;    // block 0: that entry (its times are in ts)
+    double limit;      // links from which a move pulls
+    int all;           // this move is all-green
+    double2 mm, apr;   // this move's totals: sum m, sum |m|; ||C||_1, sum v^r
+    unsigned long long rsv;  // its links and green nodes, packed
+    long long n_pieces;  // its pieces of long rows
+    double mean;       // sum v^r / N of the cash the statistics were taken of
+    unsigned long long now;  // block 0's timer when they were taken
     // TOPFRAC: this move's radix select
     unsigned long long tk_prefix;
     long long tk_remain;
     unsigned int tk_pass;  // passes made by the solve so far (histogram rotation)
 };
 
-// This move's schedule, threshold and schedule constants from the
-// statistics l1 = ||C||_1 and sumr = sum v^r (thread 0; the same in every
-// block).
-__device__ __forceinline__ void sweep_theta(SweepCtl& sc, const Control& ctl, int n, double l1, double sumr) {
+// A move whose predecessor used at least this share of the links from which
+// a move pulls writes its dense moved cash while it selects; one that pulls
+// without having done so sets it from the lists (two passes more, once: its
+// successor is expected to pull).
+constexpr double kDenseShare = 0.5;
+
+// x / y and u / v in the time of one FP64 division (0.3 us): the even lanes
+// of warp 0 take the first, the odd ones the second. Every lane of warp 0
+// calls it; all of them get both.
+__device__ __forceinline__ double2 two_ratios(double x, double y, double u, double v) {
+    const bool odd = (threadIdx.x & 1u) != 0u;
+    const double q = (odd ? u : x) / (odd ? v : y);
+    return make_double2(__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1));
+}
+
+// mean^(1/r) for r >= 2, out of line (rare; pow is large).
+__device__ __noinline__ double root_r(double mean, int r) { return pow(mean, 1.0 / r); }
+
+// What thread 0 decides for the next move from the statistics of a cash
+// (l1 = ||C||_1, mean = sum v^r / N): its schedule, threshold and schedule
+// constants, and how it will be made.
+template <typename T>
+__device__ __forceinline__ void set_move(SweepCtl& sc, const Control& ctl, MoveView<T>& mv, SweepSmem<T>& sm,
+                                         const unsigned char* masks, int n, double l1, double mean) {
     const int r = ctl.r;
     int sched = ctl.sched;
     if (ctl.safety_every > 0 && ((sc.solve_moves + 1) % ctl.safety_every) == 0) sched = SCHED_ALL_GREEN;
     double theta = 0.0;
-    if (sched == SCHED_THRESHOLD || sched == SCHED_LINK) {
-        const double mean = sumr / (double)n;
-        theta = ctl.theta_arg > 0.0 ? ctl.theta_arg
-                                    : (r == 1 ? ctl.theta_scale * mean : ctl.theta_scale * pow(mean, 1.0 / r));
-    }
+    if (sched == SCHED_THRESHOLD || sched == SCHED_LINK)
+        theta = ctl.theta_arg > 0.0 ? ctl.theta_arg : ctl.theta_scale * (r == 1 ? mean : root_r(mean, r));
     sc.sched = sched;
     sc.theta = theta;
-    sc.ax = sched_aux(ctl, n, sc.moves, l1, sched);
-    sc.mask_off = (sched == SCHED_MASK) ? (sc.mask_cursor % ctl.n_masks) * (long long)n : 0;
     sc.theta_f = (sched == SCHED_LINK) ? __double2float_rn(theta) : __double2float_ru(theta);
+    if (sched == SCHED_BLOCK_RR || sched == SCHED_PC) sc.ax = sched_aux(ctl, n, sc.moves, l1, sched);
+    mv.sched = sched;
+    mv.th = std::is_same<T, float>::value ? (T)sc.theta_f : (T)sc.theta;
+    mv.mask = (sched == SCHED_MASK) ? masks + (sc.mask_cursor % ctl.n_masks) * (long long)n : nullptr;
+    mv.acc = ctl.theta_lag && sc.have_lag;
+    sc.all = sched == SCHED_ALL_GREEN ? 1 : 0;
+    mv.dense = sc.all || (double)sc.edges >= kDenseShare * sc.limit;
+    sm.next_group = sm.n_list = sm.next_list = sm.n_mid = sm.next_mid = 0;
 }
 
-// The decisions of a move of the stale threshold that need no new
-// statistics (thread 0): degenerate history, max_steps, time; the threshold
-// from the statistics of the cash before the previous move. Every input is
-// known once the previous move has read its totals, so this runs while the
-// block waits at that move's last barrier.
-__device__ __forceinline__ void sweep_lag_control(SweepCtl& sc, const Control& ctl, int n) {
-    sc.iters++;
-    int stop = -1;
-    const bool degenerate = !(fabs(sc.hsum) > 1e-12 * sc.habs) || sc.habs == 0.0;
-    if (degenerate) stop = ST_DEGENERATE;
-    else if (sc.solve_moves >= ctl.max_steps) stop = ST_NOCONV;
-    else if ((double)(sc.lag_now - sc.t_start) > ctl.time_limit_ns || sc.iters > ctl.max_iters)
-        stop = ST_TIMEOUT;
-    sc.lag_stop = stop;
-    sc.leave = stop >= 0 ? 1 : 0;
-    sc.want_refresh = 0;
-    sweep_theta(sc, ctl, n, sc.lag_l1, sc.lag_sumr);
-    sc.pre_done = 1;
+// Block 0, thread 0: what other kernels and the host read of the last move.
+// Written while the block waits at the next barrier or before it returns.
+__device__ __forceinline__ void write_owed(SweepCtl& sc, DevState* st, MoveRecord* log) {
+    if (!sc.owed) return;
+    sc.owed = 0;
+    st->theta = sc.rec.theta;
+    st->green = sc.rec.green;
+    st->edges = sc.rec.edges;
+    st->hsum = sc.hsum;
+    st->habs = sc.habs;
+    st->last_mabs = sc.mabs;
+    st->moves = sc.moves;
+    st->solve_moves = sc.solve_moves;
+    st->tot_green = sc.tot_green;
+    st->tot_edges = sc.tot_edges;
+    st->push_moves = sc.push_moves;
+    st->pull_moves = sc.pull_moves;
+    st->fresh = 0;
+    st->skip_move = 0;
+    st->mask_cursor = sc.mask_cursor;
+    st->mode = sc.rec.mode;
+    const unsigned long long* ts = sc.ts[sc.tb ^ 1];
+    for (int q = 0; q < 6; ++q) sc.rec.phase_us[q] = (float)(ts[q + 1] - ts[q]) * 1e-3f;
+    log[sc.rec.move % kLogCap] = sc.rec;
 }
 
 __device__ __forceinline__ void clear_slot(SweepSlot* o) {
@@ -860,11 +925,65 @@ __device__ __forceinline__ void clear_slot(SweepSlot* o) {
     o->mabs = 0.0;
     o->reserve = 0ull;
     o->chunk_next = 0ull;
-    o->range_next = 0ull;
+    o->pieces = 0ull;
+}
+
+__device__ __forceinline__ int rot3(int q) { return q == 2 ? 0 : q + 1; }
+
+// Sums of four values a lane over the warp: the total of v[k] ends in lanes
+// 8 k to 8 k + 7. Six additions in a row of five steps, where four sums one
+// by one take twenty (an FP64 addition holds the SM's FP64 pipe for 16
+// cycles).
+template <typename T>
+__device__ __forceinline__ T warp_sum4(const T (&v)[4]) {
+    const int lane = threadIdx.x & 31;
+    const bool hi = (lane & 16) != 0, hh = (lane & 8) != 0;
+    T a = hi ? v[2] : v[0], b = hi ? v[3] : v[1];
+    a += __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
+    b += __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 16);
+    T x = hh ? b : a;
+    x += __shfl_xor_sync(0xffffffffu, hh ? a : b, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// The block's sums of a pass into the move's slot: sum m, sum |m|, ||C||_1,
+// sum v^r in the cash type, the links and green nodes packed (green: the
+// block's count of them, NULL for none); one FP64 (or
+// 64-bit) addition per total that is not zero. A grid barrier follows every
+// call, so the scratch is free again.
+template <typename T>
+struct PubSmem {
+    T v[4][kSweepWarps];
+    unsigned long long r[kSweepWarps];
+};
+template <typename T>
+__device__ __forceinline__ void publish(const NodeAcc<T>& acc, SweepSlot* sl, PubSmem<T>& ps, bool stamp,
+                                        const int* green = nullptr) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    {
+        const T v[4] = {acc.m, acc.ma, acc.a, acc.pr};
+        const T x = warp_sum4(v);
+        const unsigned long long r = warp_sum(acc.edges);
+        if ((lane & 7) == 0) ps.v[lane >> 3][wid] = x;
+        if (lane == 0) ps.r[wid] = r;
+    }
+    __syncthreads();
+    if (wid == 0) {
+        const T v[4] = {ps.v[0][lane], ps.v[1][lane], ps.v[2][lane], ps.v[3][lane]};
+        const T x = warp_sum4(v);
+        double* out = lane < 8 ? &sl->msum : (lane < 16 ? &sl->mabs : (lane < 24 ? &sl->a : &sl->pr));
+        if ((lane & 7) == 0 && x != T(0)) atomicAdd(out, (double)x);
+        if (lane == 0 && blockIdx.x == 0 && stamp) sl->tstamp = globaltimer();
+    } else if (wid == 1) {
+        const unsigned long long r = (warp_sum(ps.r[lane]) << kCountBits) + (green ? (unsigned int)*green : 0u);
+        if (lane == 0 && r) atomicAdd(&sl->reserve, r);
+    }
 }
 
 template <typename T, bool kHasW>
-__global__ void __launch_bounds__(kThreads, kSweepMinBlocks) k_sweep(SweepArgs<T> A) {
+__global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
     DevState* st = A.st;
     SweepState* sw = A.sw;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
@@ -872,22 +991,32 @@ __global__ void __launch_bounds__(kThreads, kSweepMinBlocks) k_sweep(SweepArgs<T
         if (A.use_cond && lead) cudaGraphSetConditional(A.cond_loop, 0u);
         return;
     }
-    __shared__ SweepSmem<T> sm;
-    __shared__ T tscratch[32];
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    SweepSmem<T>& sm = *reinterpret_cast<SweepSmem<T>*>(dyn_smem);
+    __shared__ PubSmem<T> ps;
     __shared__ SweepCtl sc;
+    __shared__ MoveView<T> mv;
     // The solve's parameters, copied once: after every barrier a global read
-    // would go to L2 again (and 600 blocks would queue on the same lines).
+    // would go to L2 again.
     __shared__ Control ctl;
     __shared__ double s_l1_refresh;
+    __shared__ unsigned long long s_limit_ns;  // the solve's time limit
     {
         const unsigned int* src = reinterpret_cast<const unsigned int*>(&st->ctl);
         unsigned int* dst = reinterpret_cast<unsigned int*>(&ctl);
         for (int k = threadIdx.x; k < (int)(sizeof(Control) / 4); k += blockDim.x) dst[k] = src[k];
-        if (threadIdx.x == 0) s_l1_refresh = st->l1_refresh;
+        for (int k = threadIdx.x; k < kHubSlots; k += blockDim.x) {
+            sm.hot.hub[k] = A.n_hubs ? __ldg(A.hubs + k) : -1;
+            sm.hot.hot[k] = 0.0;
+        }
+        sm.hot.one[threadIdx.x] = {};
     }
+    __syncthreads();
     const int n = A.n;
-    constexpr bool kF32 = std::is_same<T, float>::value;
     if (threadIdx.x == 0) {
+        s_l1_refresh = st->l1_refresh;
+        // an integer number of ns exceeds the limit when it exceeds its floor
+        s_limit_ns = ctl.time_limit_ns < 9e18 ? (unsigned long long)ctl.time_limit_ns : ~0ull;
         sc.moves = st->moves;
         sc.solve_moves = st->solve_moves;
         sc.iters = st->iters;
@@ -896,6 +1025,7 @@ __global__ void __launch_bounds__(kThreads, kSweepMinBlocks) k_sweep(SweepArgs<T
         sc.tot_edges = st->tot_edges;
         sc.push_moves = st->push_moves;
         sc.pull_moves = st->pull_moves;
+        sc.edges = st->edges;  // the last move's (0 at the start of a solve)
         sc.hsum = st->hsum;
         sc.habs = st->habs;
         sc.t_start = st->t_start;
@@ -907,142 +1037,170 @@ __global__ void __launch_bounds__(kThreads, kSweepMinBlocks) k_sweep(SweepArgs<T
         // gives the count at the start of this launch.
         const unsigned long long arr = ld_acquire_u64(&sw->bar.arrived);
         sc.target = arr - arr % gridDim.x;
-        sc.p = (int)(sw->bar.parity & 1u);
+        sc.p = (int)(sw->bar.parity % 3u);
         sc.tk_pass = sw->bar.tk_pass;
-        sc.have_lag = 0;
-        sc.stop_after = -1;
-        sc.pre_done = 0;
+        sc.limit = ctl.pull_crossover * (double)ctl.nnz;
+        sc.l1 = sc.sumr = sc.mean = 0.0;
+        sc.have_lag = sc.leave = sc.made = sc.owed = sc.want_refresh = sc.tb = 0;
+        sc.stop = -1;
+        sc.ts[0][0] = globaltimer();
+        mv.mask = nullptr;
+        mv.th = T(0);
+        mv.sched = ctl.sched;
+        mv.r = ctl.r;
+        mv.link = ctl.sched == SCHED_LINK;
+        mv.acc = mv.dense = false;
+        sm.next_group = 0;
     }
     __syncthreads();
     // Test of the bounded wait: the last block leaves without arriving, so
     // the others' first barrier wait runs out.
     if (ctl.test_skip_barrier && blockIdx.x == gridDim.x - 1 && gridDim.x > 1) return;
 
-    for (;;) {
-        SweepSlot* sl = &sw->slot[sc.p];
-        if (lead) sc.ts[0] = globaltimer();
-        // A move of the stale threshold (after the first of the launch)
-        // skips the statistics pass and its barrier: its select takes the
-        // statistics of the cash before the previous move and gathers its
-        // own cash's for the stop test.
-        const bool lagged = ctl.theta_lag && sc.have_lag;
-        if (!lagged) {
-        // ---------------------------------------------------------- stats
-        {
-            const bool link = ctl.sched == SCHED_LINK;
-            T a = T(0), s = T(0), pr = T(0);
-            stats_slice<T, true>(A.c, A.ideg, n, link, ctl.r, A.vec_ok,
-                                 blockIdx.x * (long long)blockDim.x + threadIdx.x,
-                                 (long long)gridDim.x * blockDim.x, a, s, pr);
-            const T ba = block_sum(a, tscratch);
-            const T bs = block_sum(s, tscratch);
-            const T bp = block_sum(pr, tscratch);
-            if (threadIdx.x == 0) {
-                if (ba != T(0)) atomicAdd(&sl->a, (double)ba);
-                if (bs != T(0)) atomicAdd(&sl->s, (double)bs);
-                if (bp != T(0)) atomicAdd(&sl->pr, (double)bp);
-                if (blockIdx.x == 0) sl->tstamp = globaltimer();
-            }
+    auto pow_share = [&]() {
+        int lo, hi, group;
+        block_span<T>(n, lo, hi, group);
+        return pow_sum<T>(A.c, mv.link ? A.ideg : nullptr, lo, hi, mv.r);
+    };
+    // Block 0's duties of the last move, while it waits at a barrier.
+    auto owed = [&]() {
+        if (blockIdx.x == 0) write_owed(sc, st, A.log);
+    };
+    // The end of a move (thread 0, while its block waits at the move's last
+    // barrier): the stop test and the re-derivation triggers of the stale
+    // threshold, the solve's totals, and with the stale threshold the next
+    // move's decisions.
+    auto end_move = [&]() {
+        const double l1 = sc.apr.x;
+        const double sumr = (ctl.r == 1 && !mv.link) ? l1 : sc.apr.y;
+        long long green = (long long)(sc.rsv & ((1ull << kCountBits) - 1ull));
+        long long edges = (long long)(sc.rsv >> kCountBits);
+        if (sc.all) {
+            green = n;
+            edges = ctl.nnz;
         }
-        if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts + 1 : nullptr)) break;
-
-        // -------------------------------------------------------- control
-        if (threadIdx.x == 0) {
-            if (blockIdx.x == 0) clear_slot(&sw->slot[sc.p ^ 1]);
-            const int r = ctl.r;
-            const bool link = ctl.sched == SCHED_LINK;
-            const double2 apr = ldcg_pair(&sl->a);
-            const double2 rts = ldcg_pair(&sl->reserve);
-            const double sum = __ldcg(&sl->s);
-            const double l1 = apr.x;
-            const double sumr = (r == 1 && !link) ? l1 : apr.y;
-            sc.l1 = l1;
-            const unsigned long long now = (unsigned long long)__double_as_longlong(rts.y);
-            if (sc.iters == 0) sc.t_start = now;
-            sc.iters++;
-            int stop = -1;
-            bool skip = false, want_refresh = false;
-            const bool degenerate = !(fabs(sc.hsum) > 1e-12 * sc.habs) || sc.habs == 0.0;
+        if (mv.acc) {
+            // this move's cash C_t (gathered by its pass) against H_t 1; the
+            // move is made whatever the tests say
             const bool converged = sc.moves >= 1 && l1 / fabs(sc.hsum) < ctl.tol;
-            if (degenerate) {
-                stop = ST_DEGENERATE;
-            } else if (converged) {
-                if (ctl.mixed && !sc.fresh) {
-                    want_refresh = true;  // re-derive, then test again
-                    skip = true;
-                } else {
-                    stop = ST_OK;
-                }
-            } else if (sc.solve_moves >= ctl.max_steps) {
-                stop = ST_NOCONV;
-            } else if ((double)(now - sc.t_start) > ctl.time_limit_ns || sc.iters > ctl.max_iters) {
-                stop = ST_TIMEOUT;
+            bool want_refresh = false;
+            if (converged) {
+                if (ctl.mixed && !sc.fresh) want_refresh = true;  // re-derive, then test again
+                else sc.stop = ST_OK;
+            } else if (ctl.mixed && ((ctl.refresh_factor > 0.0 && l1 < ctl.refresh_factor * s_l1_refresh) ||
+                                     cash_stalled(l1, sc.stall_mark, sc.stall_count, ctl.stall_moves))) {
+                want_refresh = true;
             }
-            if (stop < 0 && !skip && ctl.mixed &&
-                ((ctl.refresh_factor > 0.0 && l1 < ctl.refresh_factor * s_l1_refresh) ||
-                 cash_stalled(l1, sc.stall_mark, sc.stall_count, ctl.stall_moves)))
-                want_refresh = true;  // after this move
-            sc.leave = (stop >= 0 || skip) ? 1 : 0;
             sc.want_refresh = want_refresh ? 1 : 0;
-            sweep_theta(sc, ctl, n, l1, sumr);
-            // the next move of the stale threshold takes these statistics
-            sc.lag_l1 = l1;
-            sc.lag_sumr = sumr;
-            sc.lag_now = now;
-            if (blockIdx.x == 0) {
-                st->l1 = l1;
-                st->sum = sum;
-                st->sumr = sumr;
-                st->iters = sc.iters;
-                st->t_start = sc.t_start;
-                st->stall_mark = sc.stall_mark;
-                st->stall_count = sc.stall_count;
-                if (sc.leave) {
-                    st->mode = MODE_NONE;
-                    sw->bar.parity = (unsigned int)(sc.p ^ 1);
-                    sw->bar.tk_pass = sc.tk_pass;
-                    if (stop >= 0) {
-                        st->done = 1;
-                        st->status = stop;
+            sc.l1 = l1;
+            sc.sumr = sumr;
+            sc.mean = sumr / (double)n;
+        }
+        sc.made = 1;
+        sc.hsum += sc.mm.x;
+        sc.habs += sc.mm.y;
+        sc.mabs = sc.mm.y;
+        sc.moves++;
+        sc.solve_moves++;
+        sc.tot_green += green;
+        sc.tot_edges += edges;
+        sc.fresh = 0;
+        if (sc.sched == SCHED_MASK) sc.mask_cursor++;
+        if (sc.mode == MODE_PUSH) sc.push_moves++;
+        if (sc.mode == MODE_PULL) sc.pull_moves++;
+        sc.edges = edges;
+        if (blockIdx.x == 0) {
+            sc.rec.move = sc.moves - 1;
+            sc.rec.green = green;
+            sc.rec.edges = edges;
+            sc.rec.mode = sc.mode;
+            sc.rec.pad = 0;
+            sc.rec.theta = sc.theta;
+            sc.rec.l1 = sc.l1;
+            sc.rec.hsum = sc.hsum;
+            sc.owed = 1;
+        }
+        sc.p = rot3(sc.p);
+        sm.next_group = 0;
+        if (sc.stop >= 0 || sc.want_refresh) {
+            sc.leave = 1;
+        } else if (ctl.theta_lag) {
+            // the tests that need no new statistics; the threshold from the
+            // statistics just read
+            sc.have_lag = 1;
+            sc.iters++;
+            const bool degenerate = !(fabs(sc.hsum) > 1e-12 * sc.habs) || sc.habs == 0.0;
+            if (degenerate) sc.stop = ST_DEGENERATE;
+            else if (sc.solve_moves >= ctl.max_steps) sc.stop = ST_NOCONV;
+            else if (sc.now - sc.t_start > s_limit_ns || sc.iters > ctl.max_iters) sc.stop = ST_TIMEOUT;
+            sc.leave = sc.stop >= 0 ? 1 : 0;
+            set_move<T>(sc, ctl, mv, sm, A.masks, n, sc.l1, sc.mean);
+        }
+    };
+
+    for (;;) {
+        // A move of the stale threshold (after the first of the launch) has
+        // no statistics pass and no barrier for it: its threshold comes from
+        // the statistics of the cash before the previous move, and it
+        // gathers its own cash's for the stop test.
+        if (!(ctl.theta_lag && sc.have_lag)) {
+            // ------------------------------------------ stats and control
+            {
+                NodeAcc<T> acc = kNoAcc<T>;
+                node_pass<T, kHasW, PASS_STATS>(A, mv, sc.ax, sm, acc);
+                if (mv.r > 2) acc.pr = pow_share();
+                publish<T>(acc, &sw->slot[sc.p], ps, true);
+            }
+            auto control = [&]() {
+                const SweepSlot* sl = &sw->slot[sc.p];
+                const double2 apr = ldcg_pair(&sl->a);
+                const double2 rts = ldcg_pair(&sl->reserve);
+                const double l1 = apr.x;
+                const double sumr = (ctl.r == 1 && !mv.link) ? l1 : apr.y;
+                const double2 q = two_ratios(l1, fabs(sc.hsum), sumr, (double)n);
+                if (threadIdx.x != 0) return;
+                // (every block is done with the last move's slot; a launch
+                // that ends here has no move that would clear it)
+                if (blockIdx.x == 0) clear_slot(&sw->slot[rot3(rot3(sc.p))]);
+                sc.l1 = l1;
+                sc.sumr = sumr;
+                sc.mean = q.y;
+                sc.now = (unsigned long long)__double_as_longlong(rts.y);
+                if (sc.iters == 0) sc.t_start = sc.now;
+                sc.iters++;
+                bool skip = false, want_refresh = false;
+                const bool degenerate = !(fabs(sc.hsum) > 1e-12 * sc.habs) || sc.habs == 0.0;
+                const bool converged = sc.moves >= 1 && q.x < ctl.tol;
+                if (degenerate) {
+                    sc.stop = ST_DEGENERATE;
+                } else if (converged) {
+                    if (ctl.mixed && !sc.fresh) {
+                        want_refresh = true;  // re-derive, then test again
+                        skip = true;
                     } else {
-                        st->want_refresh = 1;
-                        st->skip_move = 1;
+                        sc.stop = ST_OK;
                     }
-                    if (A.use_cond) {
-                        if (stop >= 0) cudaGraphSetConditional(A.cond_loop, 0u);
-                        if (ctl.mixed) cudaGraphSetConditional(A.cond_refresh, stop >= 0 ? 0u : 1u);
-                    }
+                } else if (sc.solve_moves >= ctl.max_steps) {
+                    sc.stop = ST_NOCONV;
+                } else if (sc.now - sc.t_start > s_limit_ns || sc.iters > ctl.max_iters) {
+                    sc.stop = ST_TIMEOUT;
                 }
-            }
-        }
-        __syncthreads();
-        if (sc.leave) return;
-        } else {
-        // ------------------------------------- control (stale threshold)
-        // the tests that need no new statistics, the threshold from the
-        // previous move's
-        if (lead) sc.ts[1] = sc.ts[2] = sc.ts[0];
-        if (threadIdx.x == 0) {
-            if (!sc.pre_done) sweep_lag_control(sc, ctl, n);
-            sc.pre_done = 0;
-            const int stop = sc.lag_stop;
-            if (blockIdx.x == 0 && stop >= 0) {
-                // this move's slot is still clear: the next launch may take it
-                st->iters = sc.iters;
-                st->mode = MODE_NONE;
-                sw->bar.parity = (unsigned int)sc.p;
-                sw->bar.tk_pass = sc.tk_pass;
-                st->done = 1;
-                st->status = stop;
-                if (A.use_cond) {
-                    cudaGraphSetConditional(A.cond_loop, 0u);
-                    if (ctl.mixed) cudaGraphSetConditional(A.cond_refresh, 0u);
+                if (sc.stop < 0 && !skip && ctl.mixed &&
+                    ((ctl.refresh_factor > 0.0 && l1 < ctl.refresh_factor * s_l1_refresh) ||
+                     cash_stalled(l1, sc.stall_mark, sc.stall_count, ctl.stall_moves)))
+                    want_refresh = true;  // after this move
+                sc.want_refresh = want_refresh ? 1 : 0;
+                if (sc.stop >= 0 || skip) {
+                    sc.leave = skip ? 2 : 1;
+                    sc.p = rot3(sc.p);  // this slot holds the statistics
                 }
-            }
+                set_move<T>(sc, ctl, mv, sm, A.masks, n, l1, q.y);
+            };
+            if (!grid_barrier_with(&sw->bar, sc.target, ctl.barrier_limit_ns,
+                                   blockIdx.x == 0 ? sc.ts[sc.tb] + 1 : nullptr, owed, control))
+                goto aborted;
         }
-        __syncthreads();
-        if (sc.leave) return;
-        }
+        if (sc.leave) break;
 
         // ------------------------------------------------ top-k threshold
         // TOPFRAC: theta = the exact k-th largest |C| (k = ceil(f N)), one
@@ -1057,13 +1215,12 @@ __global__ void __launch_bounds__(kThreads, kSweepMinBlocks) k_sweep(SweepArgs<T
                 sc.tk_remain = k;
             }
             __syncthreads();
-            bool bar_ok = true;
             for (int hi = KeyOf<T>::bits; hi > 0; hi -= kRadixBits) {
                 const int width = hi >= kRadixBits ? kRadixBits : hi;
                 const int shift = hi - width;
                 const unsigned int q = sc.tk_pass;
                 sweep_radix_count<T>(A.c, n, sw->tk_hist[q % 3u], sc.tk_prefix, shift, width, sm.hist);
-                if (!(bar_ok = grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns))) break;
+                if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns)) goto aborted;
                 if (blockIdx.x == 0) {
                     unsigned int* old = sw->tk_hist[(q + 2u) % 3u];
                     for (int b = threadIdx.x; b < kRadixBins; b += blockDim.x) old[b] = 0u;
@@ -1072,184 +1229,111 @@ __global__ void __launch_bounds__(kThreads, kSweepMinBlocks) k_sweep(SweepArgs<T
                 if (threadIdx.x == 0) sc.tk_pass = q + 1u;
                 __syncthreads();
             }
-            if (!bar_ok) break;
             if (threadIdx.x == 0) {
                 sc.theta = KeyOf<T>::value(sc.tk_prefix);
                 sc.theta_f = __double2float_ru(sc.theta);
+                mv.th = std::is_same<T, float>::value ? (T)sc.theta_f : (T)sc.theta;
             }
             __syncthreads();
         }
 
         // --------------------------------------------------------- select
         {
-            const int sched = sc.sched;
-            const T th = kF32 ? (T)sc.theta_f : (T)sc.theta;
-            const unsigned char* mask = (sched == SCHED_MASK) ? A.masks + sc.mask_off : nullptr;
-            const SchedAux& ax = sc.ax;
-            double bmsum, bmabs, ba, bpr;
-            const bool link = ctl.sched == SCHED_LINK;
-            sweep_select<T>(A, sched, th, mask, ax, sl, sm.sel, lagged, link, ctl.r, bmsum, bmabs, ba, bpr);
-            if (threadIdx.x == 0) {
-                if (bmsum != 0.0) atomicAdd(&sl->msum, bmsum);
-                if (bmabs != 0.0) atomicAdd(&sl->mabs, bmabs);
-                if (lagged) {
-                    if (ba != 0.0) atomicAdd(&sl->a, ba);
-                    if (bpr != 0.0) atomicAdd(&sl->pr, bpr);
-                    if (blockIdx.x == 0) sl->tstamp = globaltimer();
-                }
+            if (mv.acc && mv.r > 2) {
+                NodeAcc<T> acc = kNoAcc<T>;
+                acc.pr = pow_share();
+                publish<T>(acc, &sw->slot[sc.p], ps, false);
+                __syncthreads();  // (the scratch is used again; the selection clears cash)
             }
+            if (threadIdx.x == 0) sm.next_group = 0;
+            if (threadIdx.x == 0) mv.n_pieces = &sw->slot[sc.p].pieces;
+            __syncthreads();
+            NodeAcc<T> acc = kNoAcc<T>;
+            if (sc.all) node_pass<T, kHasW, PASS_ALL>(A, mv, sc.ax, sm, acc);
+            else node_pass<T, kHasW, PASS_SELECT>(A, mv, sc.ax, sm, acc);
+            publish<T>(acc, &sw->slot[sc.p], ps, mv.acc, &sm.n_list);
         }
-        if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts + 3 : nullptr)) break;
-
-        // ---------------------------------------------------- choose move
-        if (threadIdx.x == 0) {
-            const int sched = sc.sched;
-            // every total of the move in one round of paired loads
-            const double2 mm = ldcg_pair(&sl->msum);
-            const double2 rts = ldcg_pair(&sl->reserve);
-            const double2 apr = ldcg_pair(&sl->a);
-            const unsigned long long rsv = (unsigned long long)__double_as_longlong(rts.x);
-            long long green = (long long)(rsv & ((1ull << kCountBits) - 1ull));
-            long long edges = (long long)(rsv >> kCountBits);
-            if (sched == SCHED_ALL_GREEN) {
-                green = n;
-                edges = ctl.nnz;
-            }
-            const double ms = mm.x, ma = mm.y;
-            if (lagged) {
-                // stop test and re-derivation triggers on this move's cash
-                // C_t (gathered by the select), against H_t 1; the move is
-                // made whatever they say
-                const int r = ctl.r;
-                const bool link = ctl.sched == SCHED_LINK;
-                const double l1 = apr.x;
-                const double sumr = (r == 1 && !link) ? l1 : apr.y;
-                const unsigned long long now = (unsigned long long)__double_as_longlong(rts.y);
-                const bool converged = sc.moves >= 1 && l1 / fabs(sc.hsum) < ctl.tol;
-                bool want_refresh = false;
-                if (converged) {
-                    if (ctl.mixed && !sc.fresh) want_refresh = true;  // re-derive, then test again
-                    else sc.stop_after = ST_OK;
-                } else if (ctl.mixed &&
-                           ((ctl.refresh_factor > 0.0 && l1 < ctl.refresh_factor * s_l1_refresh) ||
-                            cash_stalled(l1, sc.stall_mark, sc.stall_count, ctl.stall_moves))) {
-                    want_refresh = true;
-                }
-                sc.want_refresh = want_refresh ? 1 : 0;
-                sc.l1 = l1;
-                sc.lag_l1 = l1;
-                sc.lag_sumr = sumr;
-                sc.lag_now = now;
-                if (blockIdx.x == 0) {
-                    st->l1 = l1;
-                    st->sumr = sumr;
-                    st->iters = sc.iters;
-                    st->stall_mark = sc.stall_mark;
-                    st->stall_count = sc.stall_count;
-                    // every block is done with the other slot (the last move's)
-                    clear_slot(&sw->slot[sc.p ^ 1]);
-                }
-            }
-            if (ctl.theta_lag) sc.have_lag = 1;
-            sc.hsum += ms;
-            sc.habs += ma;
-            sc.moves++;
-            sc.solve_moves++;
-            sc.tot_green += green;
-            sc.tot_edges += edges;
-            sc.fresh = 0;
-            if (sched == SCHED_MASK) sc.mask_cursor++;
-            int mode;
-            if (green == 0) mode = MODE_NONE;
-            else if (sched == SCHED_ALL_GREEN || (double)edges >= ctl.pull_crossover * (double)ctl.nnz)
-                mode = MODE_PULL;
-            else
-                mode = MODE_PUSH;
-            if (mode == MODE_PUSH) sc.push_moves++;
-            if (mode == MODE_PULL) sc.pull_moves++;
-            sc.mode = mode;
-            sc.green = green;
-            sc.edges = edges;
-            if (blockIdx.x == 0) {
-                st->theta = sc.theta;
-                st->theta_f = sc.theta_f;
-                st->green = green;
-                st->edges = edges;
-                st->hsum = sc.hsum;
-                st->habs = sc.habs;
-                st->last_mabs = ma;
-                st->moves = sc.moves;
-                st->solve_moves = sc.solve_moves;
-                st->tot_green = sc.tot_green;
-                st->tot_edges = sc.tot_edges;
-                st->push_moves = sc.push_moves;
-                st->pull_moves = sc.pull_moves;
-                st->fresh = 0;
-                st->skip_move = 0;
-                st->mask_cursor = sc.mask_cursor;
-                st->mode = mode;
-                MoveRecord rec;
-                rec.move = sc.moves - 1;
-                rec.green = green;
-                rec.edges = edges;
-                rec.mode = mode;
-                rec.pad = 0;
-                rec.theta = sc.theta;
-                rec.l1 = st->l1;
-                rec.hsum = sc.hsum;
-                for (int q = 0; q < 4; ++q) rec.phase_us[q] = (float)(sc.ts[q + 1] - sc.ts[q]) * 1e-3f;
-                rec.phase_us[4] = rec.phase_us[5] = 0.f;
-                A.log[rec.move % kLogCap] = rec;
-            }
+        {
+            auto choose = [&]() {
+                // every total of the move in one round of loads
+                SweepSlot* sl = &sw->slot[sc.p];
+                const double2 rts = ldcg_pair(&sl->reserve);
+                const double2 mm = ldcg_pair(&sl->msum);
+                const double2 apr = ldcg_pair(&sl->a);
+                const unsigned long long np = __ldcg(&sl->pieces);
+                if (threadIdx.x != 0) return;
+                const unsigned long long rsv = (unsigned long long)__double_as_longlong(rts.x);
+                if (sc.all) sc.mode = MODE_PULL;
+                else if ((rsv & ((1ull << kCountBits) - 1ull)) == 0ull) sc.mode = MODE_NONE;
+                else sc.mode = (double)(rsv >> kCountBits) >= sc.limit ? MODE_PULL : MODE_PUSH;
+                sc.rsv = rsv;
+                sc.mm = mm;
+                sc.apr = apr;
+                sc.n_pieces = (long long)np;
+                if (mv.acc) sc.now = (unsigned long long)__double_as_longlong(rts.y);
+                // every block is done with the last move's slot
+                if (blockIdx.x == 0) clear_slot(&sw->slot[rot3(rot3(sc.p))]);
+            };
+            if (!grid_barrier_with(&sw->bar, sc.target, ctl.barrier_limit_ns,
+                                   blockIdx.x == 0 ? sc.ts[sc.tb] + 3 : nullptr, owed, choose))
+                goto aborted;
         }
-        __syncthreads();
 
         // ----------------------------------------------------------- move
-        if (sc.mode == MODE_PUSH)
-            push_chunks<T, kHasW, true>(A.c, A.col, A.w, A.f_eoff, A.f_base, A.f_m, A.chunk_row,
-                                        sc.edges, sc.green, blockIdx.x, gridDim.x, sm.push,
-                                        A.hubs, &sl->chunk_next);
-        else if (sc.mode == MODE_PULL)
-            pull_tiles<T, T, kHasW, true>(A.c, A.mt, A.t_ptr, A.t_src, A.t_w, A.tile_r, A.tile_e,
-                                          A.ntiles, blockIdx.x, gridDim.x, sm.pull, &sl->chunk_next);
-        // the stale threshold's next move: its decisions while this block waits
-        if (!grid_barrier_with(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts + 5 : nullptr,
-                               [&]() {
-                                   if (ctl.theta_lag && sc.stop_after < 0 && !sc.want_refresh)
-                                       sweep_lag_control(sc, ctl, n);
-                               }))
-            break;
-        if (lead) {
-            MoveRecord* rec = A.log + ((sc.moves - 1) % kLogCap);
-            rec->phase_us[4] = (float)(sc.ts[5] - sc.ts[4]) * 1e-3f;
-            rec->phase_us[5] = (float)(sc.ts[6] - sc.ts[5]) * 1e-3f;
-        }
-        if (sc.stop_after >= 0) {
-            if (lead) {
-                st->done = 1;
-                st->status = sc.stop_after;
-                st->mode = MODE_NONE;
-                sw->bar.parity = (unsigned int)(sc.p ^ 1);
-                sw->bar.tk_pass = sc.tk_pass;
-                if (A.use_cond) {
-                    cudaGraphSetConditional(A.cond_loop, 0u);
-                    if (ctl.mixed) cudaGraphSetConditional(A.cond_refresh, 0u);
-                }
+        if (sc.mode == MODE_PUSH) {
+            push_rows<T, kHasW>(A, sm, (int)sc.n_pieces);
+            if (A.n_hubs) flush_hubs<T>(A, sm.hot);
+        } else if (sc.mode == MODE_PULL) {
+            if (!sc.all && !mv.dense) {
+                dense_from_lists<T>(A, sm);
+                if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns)) goto aborted;
             }
-            return;
+            pull_tiles<T, T, kHasW, true, kSweepThreads>(A.c, A.mt, A.t_ptr, A.t_src, A.t_w, A.tile_r, A.tile_e,
+                                                         A.ntiles, blockIdx.x, gridDim.x, sm.pull,
+                                                         &sw->slot[sc.p].chunk_next);
         }
-        if (sc.want_refresh) {
-            if (lead) {
-                st->want_refresh = 1;
-                sw->bar.parity = (unsigned int)(sc.p ^ 1);
-                sw->bar.tk_pass = sc.tk_pass;
-                if (A.use_cond) cudaGraphSetConditional(A.cond_refresh, 1u);
-            }
-            return;
+        {
+            // (the move's times stay until they are logged: the next move
+            // has the other set)
+            auto times = [&]() {
+                if (threadIdx.x != 0 || blockIdx.x != 0) return;
+                sc.tb ^= 1;
+                sc.ts[sc.tb][0] = sc.ts[sc.tb][1] = sc.ts[sc.tb][2] = sc.ts[sc.tb ^ 1][6];
+            };
+            if (!grid_barrier_with(&sw->bar, sc.target, ctl.barrier_limit_ns,
+                                   blockIdx.x == 0 ? sc.ts[sc.tb] + 5 : nullptr, end_move, times))
+                goto aborted;
         }
-        if (threadIdx.x == 0) sc.p ^= 1;
-        __syncthreads();
+        if (sc.leave) break;
     }
+    if (lead) {
+        write_owed(sc, st, A.log);
+        st->l1 = sc.l1;
+        st->sumr = sc.sumr;
+        st->iters = sc.iters;
+        st->t_start = sc.t_start;
+        st->stall_mark = sc.stall_mark;
+        st->stall_count = sc.stall_count;
+        sw->bar.parity = (unsigned int)sc.p;
+        sw->bar.tk_pass = sc.tk_pass;
+        if (sc.stop >= 0) {
+            st->done = 1;
+            st->status = sc.stop;
+            st->mode = MODE_NONE;
+        } else {
+            st->want_refresh = 1;
+            if (sc.leave == 2) {  // the last test was of a cash to re-derive: no move
+                st->skip_move = 1;
+                st->mode = MODE_NONE;
+            }
+        }
+        if (A.use_cond) {
+            if (sc.stop >= 0) cudaGraphSetConditional(A.cond_loop, 0u);
+            if (ctl.mixed) cudaGraphSetConditional(A.cond_refresh, sc.stop >= 0 ? 0u : 1u);
+        }
+    }
+    return;
+aborted:
     // A barrier wait gave up: end the solve with an error status.
     if (threadIdx.x == 0) {
         st->done = 1;
