@@ -125,6 +125,8 @@ struct rlgl_ctx {
     int n_hubs = 0;
     int hub1 = -1;        // the hub when there is one
     int* deg = nullptr;      // links of each row
+    int* rank = nullptr;     // source order of the in-link copy (see source_of); null for a batch
+    HotInfo* hot = nullptr;  // its hot front
     void* f_list = nullptr;  // the phase kernels' f_eoff and f_base; the sweep's list of green rows
     void* pieces = nullptr;  // pieces of the long green rows of a move (sweep)
     // profiling
@@ -333,7 +335,7 @@ static rlgl_status enqueue_refresh(Launch L) {
     rlgl_ctx* ctx = L.ctx;
     const int n = (int)ctx->n;
     LAUNCH(L, KC_REFRESH,
-           (k_refresh_src<<<ctx->grid_nodes, kThreads, 0, ctx->stream>>>(ctx->H, ctx->s, n,
+           (k_refresh_src<<<ctx->grid_nodes, kThreads, 0, ctx->stream>>>(ctx->H, ctx->s, n, ctx->rank,
                                                                           ctx->hsrc, ctx->st)));
     LAUNCH(L, KC_REFRESH, launch_rederive_pull(ctx));
     LAUNCH(L, KC_REFRESH,
@@ -385,13 +387,13 @@ static rlgl_status enqueue_head(Launch L, int sched, const Conds& cd) {
         LAUNCH(L, KC_SELECT,
                (k_select<T, true><<<ctx->grid_select, kThreads, 0, ctx->stream>>>(
                    (T*)ctx->c, ctx->H, ctx->s, ctx->sf, ctx->row_ptr, (const T*)ctx->ideg, ctx->masks, n,
-                   (T*)ctx->mt, ctx->f_eoff, ctx->f_base, (T*)ctx->f_m, ctx->chunk_row, ctx->st,
+                   (T*)ctx->mt, ctx->rank, ctx->f_eoff, ctx->f_base, (T*)ctx->f_m, ctx->chunk_row, ctx->st,
                    ctx->part, ctx->log, cd.mode, cd.use, bv)));
     else
         LAUNCH(L, KC_SELECT,
                (k_select<T, false><<<ctx->grid_select, kThreads, 0, ctx->stream>>>(
                    (T*)ctx->c, ctx->H, ctx->s, ctx->sf, ctx->row_ptr, (const T*)ctx->ideg, ctx->masks, n,
-                   (T*)ctx->mt, ctx->f_eoff, ctx->f_base, (T*)ctx->f_m, ctx->chunk_row, ctx->st,
+                   (T*)ctx->mt, ctx->rank, ctx->f_eoff, ctx->f_base, (T*)ctx->f_m, ctx->chunk_row, ctx->st,
                    ctx->part, ctx->log, cd.mode, cd.use, bv)));
     return RLGL_OK;
 }
@@ -459,6 +461,8 @@ static SweepArgs<T> sweep_args(rlgl_ctx* ctx, const Conds& cd) {
     a.row_ptr = ctx->row_ptr;
     a.ideg = (const T*)ctx->ideg;
     a.masks = ctx->masks;
+    a.rank = ctx->rank;
+    a.hot = ctx->hot;
     a.mt = (T*)ctx->mt;
     a.mt2 = (T*)ctx->hsrc;  // free while no re-derivation runs
     a.facc = (T*)ctx->f_m;  // the power sweep clears it at every launch
@@ -508,9 +512,9 @@ static rlgl_status enqueue_power(Launch L, const Conds& cd) {
     rlgl_ctx* ctx = L.ctx;
     const SweepArgs<T> a = sweep_args<T>(ctx, cd);
     if (ctx->has_w)
-        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_power, kThreads, 0, k_power<T, true>, a))));
+        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_power, kPowThreads, sizeof(PowSmem<T>), k_power<T, true>, a))));
     else
-        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_power, kThreads, 0, k_power<T, false>, a))));
+        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_power, kPowThreads, sizeof(PowSmem<T>), k_power<T, false>, a))));
     return RLGL_OK;
 }
 
@@ -634,25 +638,30 @@ static int sweep_grid(rlgl_ctx* ctx) {
 
 // Blocks of the power sweep: all that fit, fewer when the chain has fewer
 // merge-path tiles (and node block-iterations) than that.
-template <typename T>
-static int power_fit(rlgl_ctx* ctx) {
+template <typename T, bool kHasW>
+static int power_fit_t() {
     int nb = 0;
-    cudaError_t e = ctx->has_w
-                        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_power<T, true>, kThreads, 0)
-                        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_power<T, false>, kThreads, 0);
-    if (e != cudaSuccess) {
+    constexpr int smem = (int)sizeof(PowSmem<T>);
+    if (cudaFuncSetAttribute(k_power<T, kHasW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_power<T, kHasW>, kPowThreads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return nb;
 }
 
+template <typename T>
+static int power_fit(rlgl_ctx* ctx) {
+    return ctx->has_w ? power_fit_t<T, true>() : power_fit_t<T, false>();
+}
+
 static int power_grid(rlgl_ctx* ctx) {
     const int nb = ctx->prec == RLGL_MIXED ? power_fit<float>(ctx) : power_fit<double>(ctx);
     if (nb < 1) return 0;
     const long long fit = (long long)nb * ctx->sms;
-    long long want = ctx->ntiles;
-    const long long nodes = (ctx->n + kNodesPerIter - 1) / kNodesPerIter;
+    // (a block's warps take three times its tiles' 2048 items at once)
+    long long want = (ctx->ntiles + 2) / 3;
+    const long long nodes = (ctx->n + 4 * kPowThreads - 1) / (4 * kPowThreads);
     if (nodes > want) want = nodes;
     if (want < 1) want = 1;
     return (int)(want < fit ? want : fit);
@@ -865,7 +874,7 @@ static rlgl_status build_sweep_graph(rlgl_ctx* ctx, bool power);
 // context's buffers and grids).
 static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr, const int32_t* col,
                                  const float* w, rlgl_precision prec, rlgl_memspace src,
-                                 void* stream, rlgl_ctx** out, bool eager_graph = false) {
+                                 void* stream, rlgl_ctx** out, bool eager_graph = false, bool batch = false) {
     if (!out) return fail(nullptr, RLGL_EINVAL, "out is NULL");
     *out = nullptr;
     if (n < 1 || n >= (1ll << kCountBits)) return fail(nullptr, RLGL_EINVAL, "n=%lld out of range [1, 2^27)", (long long)n);
@@ -980,6 +989,24 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
             ctx->row_ptr, ctx->w, ctx->s, ctx->sf, ctx->chunk_row, ctx->err);
         CKL(ctx);
     }
+    // Source order of the in-link copy (a batch's pulls stay in node order):
+    // the hot sources for the all-green sweep's shared memory.
+    if (!batch) {
+        TRY(dalloc(ctx, &ctx->rank, (size_t)n));
+        TRY(dalloc(ctx, &ctx->hot, 1));
+        unsigned int* hist = nullptr;
+        TRY(dalloc(ctx, &hist, (size_t)kHotBins + 2 * (size_t)hot_cap(4)));
+        int* la = (int*)hist + kHotBins;
+        int* lb = la + hot_cap(4);
+        CK(ctx, cudaMemsetAsync(ctx->hot, 0, sizeof(HotInfo), ctx->stream));
+        CK(ctx, cudaMemsetAsync(hist, 0, kHotBins * sizeof(unsigned int), ctx->stream));
+        const int gh = grid_for(n, 1024, ctx->sms);
+        k_degree_hist<<<gh, 1024, 0, ctx->stream>>>(ctx->deg, (int)n, hist);
+        k_hot_lists<<<gh, 1024, 0, ctx->stream>>>(ctx->deg, (int)n, hist, hot_cap((int)cs), ctx->hot, ctx->rank, la, lb);
+        k_hot_swap<<<grid_for(hot_cap((int)cs), kThreads, ctx->sms), kThreads, 0, ctx->stream>>>(ctx->hot, la, lb, ctx->rank);
+        CKL(ctx);
+        dfree(ctx, hist);
+    }
     // In-link (CSC) copy: counts, scan, scatter.
     long long* cursor = nullptr;
     TRY(dalloc(ctx, &cursor, (size_t)n + 1));
@@ -1076,7 +1103,7 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
     k_chunk_rows<<<grid_for(nch + 1, kThreads, ctx->sms * 8), kThreads, 0, ctx->stream>>>(
         ctx->row_ptr, n, nnz, ctx->chunk_row);
     k_csc_scatter<<<grid_for(nch, 1, ctx->sms * 8), kThreads, 0, ctx->stream>>>(
-        ctx->row_ptr, ctx->col, ctx->w, nnz, ctx->chunk_row, cursor, ctx->t_src, ctx->t_w);
+        ctx->row_ptr, ctx->col, ctx->w, nnz, ctx->chunk_row, cursor, ctx->rank, ctx->t_src, ctx->t_w);
     CKL(ctx);
     const int gt = grid_for(ctx->ntiles + 1, kThreads, ctx->sms * 16);
     k_mp_partition<<<gt, kThreads, 0, ctx->stream>>>(ctx->t_ptr, n, nnz, ctx->ntiles, kMpItems, ctx->tile_r,
@@ -1087,12 +1114,13 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
                                                       ctx->wtile_e);
     CKL(ctx);
     CK(ctx, cudaMemsetAsync(ctx->colsum, 0, (size_t)n * sizeof(double), ctx->stream));
+    k_to_source_order<<<ctx->grid_nodes, kThreads, 0, ctx->stream>>>(ctx->s, ctx->rank, (int)n, ctx->hsrc);
     if (ctx->has_w)
         k_colsum_tiles<true><<<ctx->grid_pull, kThreads, 0, ctx->stream>>>(
-            ctx->colsum, ctx->s, ctx->t_ptr, ctx->t_src, ctx->t_w, ctx->tile_r, ctx->tile_e, ctx->ntiles);
+            ctx->colsum, ctx->hsrc, ctx->t_ptr, ctx->t_src, ctx->t_w, ctx->tile_r, ctx->tile_e, ctx->ntiles);
     else
         k_colsum_tiles<false><<<ctx->grid_pull, kThreads, 0, ctx->stream>>>(
-            ctx->colsum, ctx->s, ctx->t_ptr, ctx->t_src, ctx->t_w, ctx->tile_r, ctx->tile_e, ctx->ntiles);
+            ctx->colsum, ctx->hsrc, ctx->t_ptr, ctx->t_src, ctx->t_w, ctx->tile_r, ctx->tile_e, ctx->ntiles);
     CKL(ctx);
     if (eager_graph && ctx->params.persistent && build_sweep_graph(ctx, false) != RLGL_OK) {
         // (the first solve tries again and falls back to the phase kernels)
@@ -1176,7 +1204,7 @@ rlgl_status rlgl_create_from_state(int64_t n, int64_t nnz, const int64_t* row_pt
         return bail(fail(ctx, RLGL_ECUDA, "upload of c failed"));
     // y = H P by the residual pull (forced, measuring), then C_0 and C.
     k_set_refresh_flags<<<1, 1, 0, ctx->stream>>>(ctx->st, 1, 0);
-    k_refresh_src<<<ctx->grid_nodes, kThreads, 0, ctx->stream>>>(ctx->H, ctx->s, (int)n, ctx->hsrc, ctx->st);
+    k_refresh_src<<<ctx->grid_nodes, kThreads, 0, ctx->stream>>>(ctx->H, ctx->s, (int)n, ctx->rank, ctx->hsrc, ctx->st);
     launch_rederive_pull(ctx);
     if (ctx->prec == RLGL_MIXED)
         k_record_c0<float><<<ctx->grid_nodes, kThreads, 0, ctx->stream>>>(ctx->c0, ctx->H, ctx->y, (float*)ctx->c, (int)n, ctx->st);
@@ -1215,7 +1243,7 @@ rlgl_status rlgl_batch_create(int64_t n_chains, const int64_t* node_ptr, int64_t
     for (int64_t k = 0; k < n_chains; ++k)
         if (np[(size_t)k + 1] <= np[(size_t)k]) return fail(nullptr, RLGL_EINVAL, "chain %lld is empty", (long long)k);
     rlgl_ctx* ctx = nullptr;
-    rlgl_status s = create_common(n, nnz, row_ptr, col, w, prec, src, stream, &ctx);
+    rlgl_status s = create_common(n, nnz, row_ptr, col, w, prec, src, stream, &ctx, false, true);
     auto bail = [&](rlgl_status st) {
         if (ctx) snprintf(g_thread_err, sizeof g_thread_err, "%s", ctx->err_msg);
         rlgl_destroy(ctx);
@@ -2014,6 +2042,7 @@ int64_t rlgl_footprint(int64_t n, int64_t nnz, int32_t weighted, rlgl_precision 
     int64_t b = 0;
     b += 2 * ((n + 1) * 8 + nnz * 4 + (weighted ? nnz * 4 : 0));  // CSR and CSC
     b += n * (8 + (prec == RLGL_MIXED ? 4 : 0) + cs + 4);            // s, sf, 1/deg, deg
+    if (n_chains <= 1) b += n * 4 + (int64_t)sizeof(HotInfo);        // source order
     b += 2 * (ntiles + 1) * 8 + 2 * (nwtiles + 1) * 8;               // merge-path tiles (block, warp)
     b += n * (cs + 8 + cs + 8 + 8 + 8 + 8 + cs + 8);                 // c H mt y hsrc f_eoff f_base f_m colsum
     b += (nnz / kPushChunk + 2) * 4;                                 // chunk index
@@ -2057,7 +2086,7 @@ void rlgl_destroy(rlgl_ctx* ctx) {
     void* dev[] = {ctx->row_ptr, ctx->col, ctx->w, ctx->s, ctx->sf, ctx->ideg, ctx->t_ptr, ctx->t_src, ctx->t_w,
                    ctx->tile_r, ctx->tile_e, ctx->wtile_r, ctx->wtile_e, ctx->c, ctx->H, ctx->mt, ctx->y, ctx->hsrc, ctx->c0,
                    ctx->colsum,
-                   ctx->f_list, ctx->deg, ctx->f_m, ctx->chunk_row, ctx->part, ctx->masks,
+                   ctx->f_list, ctx->deg, ctx->rank, ctx->hot, ctx->f_m, ctx->chunk_row, ctx->part, ctx->masks,
                    ctx->err, ctx->log, ctx->st, ctx->sw, ctx->node_ptr, ctx->chain_of, ctx->cs,
                    ctx->bsums, ctx->ct_off, ctx->ct_r, ctx->ct_e, ctx->grp, ctx->bq, ctx->q_next, ctx->hubs,
                    ctx->pieces};

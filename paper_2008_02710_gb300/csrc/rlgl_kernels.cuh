@@ -266,6 +266,46 @@ __device__ __forceinline__ void red_add(double* p, double v) {
     asm volatile("red.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
 
+// Loads of links, which a pass over them reads once: first to leave the L2
+// (and not kept in L1), so that the node values gathered or added to stay.
+// (first: whether they are first to leave; else as any load)
+__device__ __forceinline__ unsigned long long stream_policy(bool first = true) {
+    unsigned long long p, q;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(q));
+    return first ? p : q;
+}
+__device__ __forceinline__ int ld_stream(const int* p, unsigned long long pol) {
+    int v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float ld_stream(const float* p, unsigned long long pol) {
+    float v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ double ld_stream(const double* p, unsigned long long pol) {
+    double v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
+    return v;
+}
+// The same for links read in short runs, whose sectors neighbouring rows
+// share: kept in L1.
+__device__ __forceinline__ int ld_run(const int* p, unsigned long long pol) {
+    int v;
+    asm("ld.global.nc.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float ld_run(const float* p, unsigned long long pol) {
+    float v;
+    asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ void red_add_stream(double* p, double v, unsigned long long pol) {
+    asm volatile("red.global.add.L2::cache_hint.f64 [%0], %1, %2;" ::"l"(p), "d"(v), "l"(pol) : "memory");
+}
+
 // Loads of data that other blocks of the same kernel may have written: from
 // L2 (ld.global.cg) when kCg, so that no stale L1 line is read.
 template <bool kCg, typename T>
@@ -846,6 +886,99 @@ __global__ void __launch_bounds__(kThreads) k_radix_pass(const T* __restrict__ c
 
 // ------------------------------------------------------------------ select
 
+// Source order. The values that pulls gather (m~, H s) are kept in source
+// order: node i's at rank[i] (null: at i), and t_src holds ranks. The nodes
+// with the most out-links, whose values are gathered the most, come first,
+// so that a kernel can keep the front of the array in shared memory
+// (k_power); all other nodes keep their place but for as many as those
+// displace, so that writes of consecutive nodes stay coalesced.
+__device__ __forceinline__ int source_of(const int* __restrict__ rank, int i) { return rank ? __ldg(rank + i) : i; }
+
+constexpr int kHotBins = 4096;      // out-degrees counted one by one below this
+constexpr int kHotMinDegree = 64;   // a hot source saves that many gathers a pull over the GPU and costs one load per SM
+struct HotInfo {
+    int thr;    // hot: out-degree >= thr
+    int count;  // hot sources
+    int na, nb; // nodes displaced, and hot nodes to move to the front
+};
+
+// Histogram of the out-degrees (those of kHotBins - 1 and more together).
+__global__ void __launch_bounds__(1024) k_degree_hist(const int* __restrict__ deg, int n, unsigned int* hist) {
+    __shared__ unsigned int h[kHotBins];
+    for (int b = threadIdx.x; b < kHotBins; b += blockDim.x) h[b] = 0u;
+    __syncthreads();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int d = deg[i];
+        if (d >= kHotMinDegree) atomicAdd(&h[min(d, kHotBins - 1)], 1u);
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < kHotBins; b += blockDim.x)
+        if (h[b]) atomicAdd(hist + b, h[b]);
+}
+
+// The hot sources (1024 threads): as many of the largest out-degrees as fit
+// `cap`, whole degrees only, none below kHotMinDegree. Hot nodes with ids
+// beyond their number go to list b, the others with smaller ids to list a
+// (equally many); every node's rank starts as its id.
+__global__ void __launch_bounds__(1024) k_hot_lists(const int* __restrict__ deg, int n,
+                                                    const unsigned int* __restrict__ hist, int cap, HotInfo* info,
+                                                    int* __restrict__ rank, int* __restrict__ la,
+                                                    int* __restrict__ lb) {
+    __shared__ int s_thr, s_count;
+    if (threadIdx.x == 0) {
+        s_thr = 0x7fffffff;
+        s_count = 0;
+    }
+    constexpr int kPer = kHotBins / 1024;
+    unsigned long long mine = 0;
+    const int top = kHotBins - 1 - (int)threadIdx.x * kPer;  // this thread's bins top, top - 1, ...
+    unsigned int h[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        h[q] = hist[top - q];
+        mine += h[q];
+    }
+    unsigned long long total;
+    unsigned long long cum = block_exscan<1024>(mine, &total);
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        cum += h[q];
+        // (the lowest bin that still fits; the count only grows downwards)
+        if (top - q >= kHotMinDegree && cum <= (unsigned long long)cap) {
+            atomicMin(&s_thr, top - q);
+            atomicMax(&s_count, (int)cum);
+        }
+    }
+    __syncthreads();
+    const int thr = s_thr, count = s_count;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        info->thr = thr;
+        info->count = count;
+    }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        rank[i] = i;
+        const bool hot = deg[i] >= thr;
+        if (hot && i >= count) lb[atomicAdd(&info->nb, 1)] = i;
+        if (!hot && i < count) la[atomicAdd(&info->na, 1)] = i;
+    }
+}
+
+__global__ void k_hot_swap(const HotInfo* __restrict__ info, const int* __restrict__ la, const int* __restrict__ lb,
+                           int* __restrict__ rank) {
+    const int m = info->na;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
+        rank[la[k]] = lb[k];
+        rank[lb[k]] = la[k];
+    }
+}
+
+// out[rank[i]] = x[i].
+__global__ void k_to_source_order(const double* __restrict__ x, const int* __restrict__ rank, int n,
+                                  double* __restrict__ out) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        out[source_of(rank, i)] = x[i];
+}
+
 // m~_i = m_i s_i, the cash a green row sends per unit of edge weight: in
 // FP64 on the FP64 path, in FP32 (with s_i rounded to FP32) on the MIXED path.
 __device__ __forceinline__ double moved_per_weight(double v, const double* s, const float*, long long i) {
@@ -864,7 +997,7 @@ __global__ void __launch_bounds__(kThreads) k_select(
     T* __restrict__ c, double* __restrict__ H, const double* __restrict__ s,
     const float* __restrict__ sf, const long long* __restrict__ row_ptr,
     const T* __restrict__ ideg, const unsigned char* __restrict__ masks, int n,
-    T* __restrict__ mt, long long* __restrict__ f_eoff, long long* __restrict__ f_base,
+    T* __restrict__ mt, const int* __restrict__ rank, long long* __restrict__ f_eoff, long long* __restrict__ f_base,
     T* __restrict__ f_m, int* __restrict__ chunk_row, DevState* st, double* part,
     MoveRecord* __restrict__ log, unsigned long long cond_mode, int use_cond, BatchView bv) {
     if (st->done || st->skip_move) return;
@@ -943,7 +1076,7 @@ __global__ void __launch_bounds__(kThreads) k_select(
                 red_add(H + i, (double)v);  // no load: the L2 adds
                 msum += v;
                 mabs += fabs(v);
-                mt[i] = v * scv[q];
+                mt[source_of(rank, (int)i)] = v * scv[q];
             }
             continue;
         }
@@ -971,7 +1104,7 @@ __global__ void __launch_bounds__(kThreads) k_select(
                     msum += v;
                     mabs += fabs(v);
                 }
-                mt[i] = mtil;
+                mt[source_of(rank, (int)i)] = mtil;
                 f_eoff[k] = e;
                 f_base[k] = rb[q] - e;
                 f_m[k] = mtil;
@@ -982,7 +1115,7 @@ __global__ void __launch_bounds__(kThreads) k_select(
                 ++k;
                 e += rdeg[q];
             } else {
-                mt[i] = T(0);
+                mt[source_of(rank, (int)i)] = T(0);
             }
         }
         if (kBatch && uni >= 0) {
@@ -1466,12 +1599,12 @@ __global__ void __launch_bounds__(kThreads) k_pull(
 
 // ------------------------------------------------------------ refresh
 
-// hsrc_i = H_i s_i (FP64), the source vector of the residual pull.
+// H_i s_i (FP64) in source order, the source vector of the residual pull.
 __global__ void k_refresh_src(const double* __restrict__ H, const double* __restrict__ s, int n,
-                              double* __restrict__ hsrc, const DevState* st) {
+                              const int* __restrict__ rank, double* __restrict__ hsrc, const DevState* st) {
     if (!(st->force_refresh || (st->want_refresh && !st->done))) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        hsrc[i] = H[i] * s[i];
+        hsrc[source_of(rank, i)] = H[i] * s[i];
 }
 
 // exact_j = C0_j + (H P)_j - H_j (Eq. recursion_H_res); residual
@@ -1818,8 +1951,8 @@ __global__ void k_chunk_rows(const long long* __restrict__ row_ptr, long long n,
 // (as in the push). Order within a CSC row is arbitrary.
 __global__ void __launch_bounds__(kThreads) k_csc_scatter(
     const long long* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ w,
-    long long nnz, const int* __restrict__ chunk_first_row, long long* cursor, int* __restrict__ t_src,
-    float* __restrict__ t_w) {
+    long long nnz, const int* __restrict__ chunk_first_row, long long* cursor, const int* __restrict__ rank,
+    int* __restrict__ t_src, float* __restrict__ t_w) {
     constexpr int kPer = kPushChunk / kThreads;
     __shared__ int s_row[kPushChunk];
     __shared__ int s_wmax[kThreads / 32];
@@ -1867,7 +2000,7 @@ __global__ void __launch_bounds__(kThreads) k_csc_scatter(
                 const long long e = e0 + le;
                 const int j = col[e];
                 const long long pos = (long long)atomicAdd((unsigned long long*)(cursor + j), 1ull);
-                t_src[pos] = k0 + s_row[le];
+                t_src[pos] = source_of(rank, k0 + s_row[le]);
                 if (w) t_w[pos] = w[e];
             }
         }

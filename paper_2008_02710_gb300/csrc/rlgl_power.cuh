@@ -33,6 +33,22 @@
 // items (FP32), 6.99 / 72.7 ms. Gathering m~ into shared memory with
 // cp.async (two tiles ahead, the warp's operands staged in dynamic shared
 // memory) was slower than loading it: 10.9 ms on R-MAT 20.
+// What bounds a move is the gathers of m~ (a random 4-byte load from L2
+// moves a 32-byte sector: 313 G/s over the GPU whatever the array's size, so
+// 60 us for R-MAT 20's 18.9 M in-links) and the instructions of the merge.
+// Measured then, us a move on R-MAT 20 / symmetrised R-MAT 24:
+//   three blocks of 256 threads an SM, no hot sources        105 / 3126
+//   one block of 768, the 14336 sources with the most out-links in shared
+//   memory (half and a third of the gathers), merge steps without branches,
+//   one load of row ends a lane, no merge for tiles inside a row  85 / 2775
+//   and the links' loads not kept in L1 and first to leave L2     71 / 2557
+// (the start of the second row on its own machine, the rest beside it). More
+// hot sources are slower: what shared memory takes is taken from L1, which
+// the loads in flight need (36864: 170 / 6690 us with the same merge as the
+// first row). A spilled register in the tile loop costs more than a larger
+// tile gives: 1024 threads at 64 registers 120 / 3880 us. A load from L2
+// into a register that a shared-memory load also writes waits for it: the
+// hot values are read first.
 // The moved cash alternates between two buffers (mt and the residual
 // source hsrc, free while no re-derivation runs). The per-move totals
 // rotate over three slots: the decision of move t reads slot q, move t adds
@@ -51,22 +67,37 @@
 namespace rlgl {
 
 constexpr int kWarpsPerBlock = kThreads / 32;
-constexpr int kPowerMinBlocks = 3;  // blocks per SM (launch bounds: up to 85 registers a thread)
+constexpr int kPowerMinBlocks = 3;  // k_rederive_pull: blocks per SM (launch bounds: up to 85 registers a thread)
+// The all-green sweep: one block of 768 threads an SM, so that the warps
+// share one copy of the hot sources and a thread has 80 registers.
+constexpr int kPowThreads = 768;
+constexpr int kPowWarps = kPowThreads / 32;
 
 // Merge-path items per lane of a warp tile: 12 for FP32 cash (384-item
 // tiles), 8 for FP64 (256-item tiles, so that a block's static shared
 // memory stays within 48 KB).
-__host__ __device__ constexpr int power_ipt(int cash_bytes) { return cash_bytes == 4 ? 12 : 8; }
+__host__ __device__ constexpr int power_ipt(int cash_bytes) { return cash_bytes == 4 ? 12 : 6; }
 
 // Shared memory of one warp of the power sweep: its merge-path tile (the
 // gathered in-link values, the row ends) and each row's in-link sum (local
-// row index).
+// row index). With FP32 cash the sums take the place of the ends: a row's
+// end is last read before the sum is there (see power_tiles).
 template <typename T>
 struct PowWarp {
     static constexpr int kItems = 32 * power_ipt((int)sizeof(T));
+    static constexpr bool kShare = sizeof(T) == sizeof(int);
     T val[kItems];
-    int end[kItems + 1];
-    T rsum[kItems];
+    int ends[kItems + 1];
+    T sums[kShare ? 1 : kItems];
+    __device__ __forceinline__ T* rsum() { return kShare ? reinterpret_cast<T*>(ends) : sums; }
+};
+
+// Hot sources kept in shared memory, and the block's dynamic shared memory.
+__host__ __device__ constexpr int hot_cap(int cash_bytes) { return cash_bytes == 4 ? 16384 : 4096; }
+template <typename T>
+struct PowSmem {
+    alignas(16) T hot[hot_cap((int)sizeof(T))];
+    PowWarp<T> warp[kPowWarps];
 };
 
 // Per-thread sums of a move: ||C_{t+1}||_1, sum C_{t+1}, sum M_t, sum |M_t|
@@ -79,11 +110,11 @@ struct PowAcc {
 // Row epilogue of an all-green move: row r's in-link sum v is C_{t+1},r;
 // old = C_t,r and sc = s_r.
 template <typename T>
-__device__ __forceinline__ void power_row_with(const SweepArgs<T>& A, T* __restrict__ mt_next, long long r, T v,
+__device__ __forceinline__ void power_row_with(const SweepArgs<T>& A, T* __restrict__ mt_next, int r, T v,
                                                T old, T sc, PowAcc<T>& acc) {
     A.c[r] = v;
-    mt_next[r] = v * sc;
-    red_add(A.H + r, (double)old);  // M_t,r joins the history (no load: the L2 adds)
+    mt_next[source_of(A.rank, r)] = v * sc;
+    red_add(A.H + r, widen(old));  // M_t,r joins the history (no load: the L2 adds)
     acc.a += fabs(v);
     acc.s += v;
     acc.m += old;
@@ -91,7 +122,7 @@ __device__ __forceinline__ void power_row_with(const SweepArgs<T>& A, T* __restr
 }
 
 template <typename T>
-__device__ __forceinline__ void power_row(const SweepArgs<T>& A, T* __restrict__ mt_next, long long r, T v,
+__device__ __forceinline__ void power_row(const SweepArgs<T>& A, T* __restrict__ mt_next, int r, T v,
                                           PowAcc<T>& acc) {
     const T old = __ldcg(A.c + r);  // C_t,r (this kernel stored it one move ago)
     const T sc = __ldg(row_scale(A.sf, A.s, T(0)) + r);
@@ -100,14 +131,14 @@ __device__ __forceinline__ void power_row(const SweepArgs<T>& A, T* __restrict__
 
 // Bounds of tile b: first row, first in-link, rows ending in it, in-links.
 struct TileB {
-    long long r0, e0;
-    int nr, ne;
+    long long e0;
+    int r0, nr, ne;
 };
 
 __device__ __forceinline__ TileB tile_bounds(const long long* __restrict__ tile_r,
                                              const long long* __restrict__ tile_e, long long b) {
     TileB t;
-    t.r0 = __ldg(tile_r + b);
+    t.r0 = (int)__ldg(tile_r + b);
     t.e0 = __ldg(tile_e + b);
     t.nr = (int)(__ldg(tile_r + b + 1) - t.r0);
     t.ne = (int)(__ldg(tile_e + b + 1) - t.e0);
@@ -116,16 +147,51 @@ __device__ __forceinline__ TileB tile_bounds(const long long* __restrict__ tile_
 
 // Segmented inclusive scan over the lanes of a warp: the running sum of val
 // restarts wherever key changes (keys >= 0 form contiguous runs).
-template <typename T>
-__device__ __forceinline__ T warp_segscan(long long key, T val) {
+template <typename T, typename K>
+__device__ __forceinline__ T warp_segscan(K key, T val) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const T y = __shfl_up_sync(0xffffffffu, val, o);
-        const long long ky = __shfl_up_sync(0xffffffffu, key, o);
+        const K ky = __shfl_up_sync(0xffffffffu, key, o);
         if (lane >= o && ky == key) val += y;
     }
     return val;
+}
+
+// The hot front of the moved cash (written by all blocks one move ago: from
+// L2) into shared memory; returns its length.
+template <typename T>
+__device__ __forceinline__ int load_hot(const SweepArgs<T>& A, const T* __restrict__ mt, PowSmem<T>& sm) {
+    const int n_hot = A.hot ? __ldg(&A.hot->count) : 0;
+    constexpr int kPer = 16 / (int)sizeof(T);
+    const int nv = n_hot / kPer;
+    const float4* src = reinterpret_cast<const float4*>(mt);
+    float4* dst = reinterpret_cast<float4*>(sm.hot);
+    for (int k = threadIdx.x; k < nv; k += 4 * kPowThreads) {
+        float4 x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (k + q * kPowThreads < nv) x[q] = __ldcg(src + k + q * kPowThreads);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (k + q * kPowThreads < nv) dst[k + q * kPowThreads] = x[q];
+    }
+    for (int k = nv * kPer + (int)threadIdx.x; k < n_hot; k += kPowThreads) sm.hot[k] = __ldcg(mt + k);
+    __syncthreads();
+    return n_hot;
+}
+
+// v = *p (from L2) where pred, else unchanged, in place.
+__device__ __forceinline__ void ld_over(float& v, const float* p, bool pred) {
+    asm volatile("{ .reg .pred q; setp.ne.s32 q, %2, 0; @q ld.global.cg.f32 %0, [%1]; }"
+                 : "+f"(v)
+                 : "l"(p), "r"((int)pred));
+}
+__device__ __forceinline__ void ld_over(double& v, const double* p, bool pred) {
+    asm volatile("{ .reg .pred q; setp.ne.s32 q, %2, 0; @q ld.global.cg.f64 %0, [%1]; }"
+                 : "+d"(v)
+                 : "l"(p), "r"((int)pred));
 }
 
 // One move's pull with the row epilogue, a warp per merge-path tile: the
@@ -137,60 +203,81 @@ __device__ __forceinline__ T warp_segscan(long long key, T val) {
 // __syncwarp. The pieces of rows that cross tile boundaries go into facc.
 template <typename T, bool kHasW>
 __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __restrict__ mt_cur,
-                                            T* __restrict__ mt_next, PowWarp<T>& ws,
+                                            T* __restrict__ mt_next, PowSmem<T>& sm, int n_hot,
                                             unsigned long long* next, PowAcc<T>& acc) {
     constexpr int kPowIpt = power_ipt((int)sizeof(T));
     const int lane = threadIdx.x & 31;
-    const long long ntiles = A.nwtiles;
-    const long long nw = (long long)gridDim.x * kWarpsPerBlock;
-    const long long w = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    const long long rounds = ntiles / nw > 2 ? ntiles / nw - 2 : 0;  // tiles taken in turn
-    const long long dyn0 = rounds * nw;                              // the first handed-out tile
+    PowWarp<T>& ws = sm.warp[threadIdx.x >> 5];
+    T* const rsum = ws.rsum();
+    const unsigned long long pol = stream_policy();
+    // (tiles: at most 2^38 / 256, an int; rows: below 2^27)
+    const int ntiles = (int)A.nwtiles;
+    const int nw = (int)gridDim.x * kPowWarps;
+    const int w = (int)blockIdx.x * kPowWarps + (int)(threadIdx.x >> 5);
+    const int dyn0 = max(ntiles / nw - 2, 0) * nw;  // tiles below are taken in turn, the rest handed out
     const T* __restrict__ scale = row_scale(A.sf, A.s, T(0));
-    unsigned long long grab = 0, g0 = 0;
-    if (lane == 0) {
-        if (rounds < 1) g0 = atomicAdd(next, 1ull);
-        if (rounds < 2) grab = atomicAdd(next, 1ull);  // turn 1
+    int b = w, grab = 0;
+    if (dyn0 == 0) {
+        if (lane == 0) b = (int)atomicAdd(next, 1ull);
+        b = __shfl_sync(0xffffffffu, b, 0);
     }
-    long long b = rounds > 0 ? w : dyn0 + (long long)__shfl_sync(0xffffffffu, g0, 0);
+    if (lane == 0 && b + nw >= dyn0) grab = (int)atomicAdd(next, 1ull);  // for the turn after
     TileB t{0, 0, 0, 0};
     int sidx[kPowIpt];
     if (b < ntiles) t = tile_bounds(A.wtile_r, A.wtile_e, b);
 #pragma unroll
     for (int q = 0; q < kPowIpt; ++q) {
         const int k = lane + q * 32;
-        sidx[q] = (b < ntiles && k < t.ne) ? __ldg(A.t_src + t.e0 + k) : -1;
+        sidx[q] = (b < ntiles && k < t.ne) ? ld_stream(A.t_src + t.e0 + k, pol) : -1;
     }
-    for (long long s = 0; b < ntiles; ++s) {
+    while (b < ntiles) {
         T oldv = T(0), scv = T(0);
         int start0;
         TileB tn{0, 0, 0, 0};
-        long long bn;
+        int bn;
         {
             // m~ of this move was written by other warps one move ago: L2
             T v[kPowIpt];
 #pragma unroll
-            for (int q = 0; q < kPowIpt; ++q) v[q] = (sidx[q] >= 0) ? __ldcg(mt_cur + sidx[q]) : T(0);
+            for (int q = 0; q < kPowIpt; ++q)
+                v[q] = (unsigned int)sidx[q] < (unsigned int)n_hot ? sm.hot[sidx[q]] : T(0);
+            // the others over them, where the value is a global load's: the
+            // shared loads come first, because a load into a register waits
+            // for an earlier one into it, and those are short
+#pragma unroll
+            for (int q = 0; q < kPowIpt; ++q) ld_over(v[q], mt_cur + sidx[q], sidx[q] >= n_hot);
 #pragma unroll
             for (int q = 0; q < kPowIpt; ++q) {
                 const int k = lane + q * 32;
                 if (kHasW && k < t.ne) asm volatile("prefetch.global.L1 [%0];" ::"l"(A.t_w + t.e0 + k));
             }
             // the next tile's bounds and sources, in flight over this tile
-            bn = s + 1 < rounds ? w + (s + 1) * nw : dyn0 + (long long)__shfl_sync(0xffffffffu, grab, 0);
-            if (bn < ntiles && s + 2 >= rounds && lane == 0) grab = atomicAdd(next, 1ull);
+            bn = b + nw;
+            if (bn >= dyn0) bn = dyn0 + __shfl_sync(0xffffffffu, grab, 0);
+            if (bn < ntiles && bn + nw >= dyn0 && lane == 0) grab = (int)atomicAdd(next, 1ull);
             if (bn < ntiles) tn = tile_bounds(A.wtile_r, A.wtile_e, bn);
 #pragma unroll
             for (int q = 0; q < kPowIpt; ++q) {
                 const int k = lane + q * 32;
-                sidx[q] = (bn < ntiles && k < tn.ne) ? __ldg(A.t_src + tn.e0 + k) : -1;
+                sidx[q] = (bn < ntiles && k < tn.ne) ? ld_stream(A.t_src + tn.e0 + k, pol) : -1;
             }
-            int re[kPowIpt];
+            if (t.nr == 0) {
+                // every item a link of one row that goes on: no merge
+                T sum = T(0);
 #pragma unroll
-            for (int q = 0; q < kPowIpt; ++q) {
-                const int k = lane + q * 32;
-                re[q] = (k < t.nr) ? (int)(__ldg(A.t_ptr + t.r0 + 1 + k) - t.e0) : 0;
+                for (int q = 0; q < kPowIpt; ++q) {
+                    const int k = lane + q * 32;
+                    sum += (kHasW && k < t.ne) ? v[q] * (T)__ldg(A.t_w + t.e0 + k) : v[q];
+                }
+                sum = warp_sum(sum);
+                if (lane == 0) atomicAdd(A.facc + t.r0, sum);
+                b = bn;
+                t = tn;
+                continue;
             }
+            // (a tile seldom holds more than 32 rows)
+            int re = 0;
+            if (lane < t.nr) re = (int)(__ldg(A.t_ptr + t.r0 + 1 + lane) - t.e0);
             start0 = (int)(__ldg(A.t_ptr + t.r0) - t.e0);
             // the epilogue's first row of this lane, read with the gathers
             if (lane < t.nr) {
@@ -201,72 +288,82 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
             for (int q = 0; q < kPowIpt; ++q) {
                 const int k = lane + q * 32;
                 if (k < t.ne) ws.val[k] = kHasW ? v[q] * (T)__ldg(A.t_w + t.e0 + k) : v[q];
-                if (k < t.nr) ws.end[k] = re[q];
             }
+            if (lane < t.nr) ws.ends[lane] = re;
+            for (int k = lane + 32; k < t.nr; k += 32) ws.ends[k] = (int)(__ldg(A.t_ptr + t.r0 + 1 + k) - t.e0);
         }
-        if (lane == 0) ws.end[t.nr] = 0x7fffffff;
+        if (lane == 0) ws.ends[t.nr] = 0x7fffffff;
         __syncwarp();
         const int total = t.nr + t.ne;
         int d = lane * kPowIpt;
-        long long rowA = -1, rowB = -1;
+        int rowA = -1, rowB = -1;  // local rows
         T accA = T(0), accB = T(0);
+        int i = 0, j = 0, row_start = 0;
         if (d < total) {
-            const int dend = min(d + kPowIpt, total);
             int lo = max(0, d - t.ne), hi = min(d, t.nr);
             while (lo < hi) {
                 int mid = (lo + hi) >> 1;
-                if (ws.end[mid] >= d - mid) hi = mid; else lo = mid + 1;
+                if (ws.ends[mid] >= d - mid) hi = mid; else lo = mid + 1;
             }
-            int i = lo, j = d - lo;
-            const int row_start = (i == 0) ? start0 : ws.end[i - 1];
+            i = lo;
+            j = d - lo;
+            row_start = (i == 0) ? start0 : ws.ends[i - 1];
+        }
+        // From here on a lane uses only the ends of rows of which it holds an
+        // item, and writes in this loop only sums of rows that lie in it
+        // whole: no other lane holds an item of those.
+        __syncwarp();
+        if (d < total) {
             bool whole = (j == row_start);  // no in-link of row i before this lane
             T sum = T(0);
-            int cnt = 0;
-            for (; d < dend; ++d) {
-                if (j < ws.end[i]) {
-                    sum += ws.val[j];
-                    ++j;
-                    ++cnt;
-                } else {
-                    if (!whole) {
-                        rowA = t.r0 + i;
+            int end = ws.ends[i], j0 = j;   // the row's end; the lane's first in-link of the row
+#pragma unroll
+            for (int q = 0; q < kPowIpt; ++q) {
+                if (d + q < total) {
+                    const bool link = j < end;
+                    if (link) sum += ws.val[j];
+                    if (!link && whole) rsum[i] = sum;  // a row with no in-link sums to zero
+                    if (!link && !whole) {
+                        rowA = i;
                         accA = sum;
-                    } else {
-                        ws.rsum[i] = sum;  // a row with no in-link sums to zero
                     }
-                    sum = T(0);
-                    cnt = 0;
-                    ++i;
-                    whole = true;
+                    if (!link) {
+                        sum = T(0);
+                        j0 = j;
+                        ++i;
+                        end = ws.ends[i];
+                        whole = true;
+                    }
+                    j += link ? 1 : 0;
                 }
             }
-            if (cnt > 0 || !whole) {
-                rowB = t.r0 + i;
+            if (j > j0 || !whole) {
+                rowB = i;
                 accB = sum;
             }
         }
         const T run = warp_segscan<T>(rowB, accB);
-        const long long pkey = __shfl_up_sync(0xffffffffu, rowB, 1);
+        const int pkey = __shfl_up_sync(0xffffffffu, rowB, 1);
         const T pval = __shfl_up_sync(0xffffffffu, run, 1);
         const bool first_split = start0 < 0;  // the tile's first row began in an earlier tile
         if (rowA >= 0) {
             T sum = accA;
             if (lane > 0 && pkey == rowA) sum += pval;
-            if (rowA == t.r0 && first_split)
-                atomicAdd(A.facc + rowA, sum);  // counted at the next tile
+            if (rowA == 0 && first_split)
+                atomicAdd(A.facc + t.r0, sum);  // finished after the barrier
             else
-                ws.rsum[rowA - t.r0] = sum;
+                rsum[rowA] = sum;
         }
         const int last = (total - 1) / kPowIpt;
-        if (lane == last && rowB >= 0) atomicAdd(A.facc + rowB, run);
+        if (lane == last && rowB >= 0) atomicAdd(A.facc + t.r0 + rowB, run);
         __syncwarp();
         // the rows that end in this tile and began in it
         for (int k = lane; k < t.nr; k += 32) {
             if (k == 0 && first_split) continue;
             if (k == lane)
-                power_row_with<T>(A, mt_next, t.r0 + k, ws.rsum[k], oldv, scv, acc);
+                power_row_with<T>(A, mt_next, t.r0 + k, rsum[k], oldv, scv, acc);
             else
-                power_row<T>(A, mt_next, t.r0 + k, ws.rsum[k], acc);
+                power_row<T>(A, mt_next, t.r0 + k, rsum[k], acc);
         }
         __syncwarp();  // the warp's shared memory is rewritten next
         b = bn;
@@ -285,7 +382,7 @@ __device__ __forceinline__ void power_split_rows(const SweepArgs<T>& A, T* __res
         if (__ldg(A.wtile_r + b + 1) == r0 || __ldg(A.t_ptr + r0) >= __ldg(A.wtile_e + b)) continue;
         const T v = __ldcg(A.facc + r0);
         A.facc[r0] = T(0);
-        power_row<T>(A, mt_next, r0, v, acc);
+        power_row<T>(A, mt_next, (int)r0, v, acc);
     }
 }
 
@@ -315,6 +412,7 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks)
     __shared__ RederiveWarp<kHasW, kIpt> sm[kWarpsPerBlock];
     RederiveWarp<kHasW, kIpt>& ws = sm[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
+    const unsigned long long pol = stream_policy();
     const long long nw = (long long)gridDim.x * kWarpsPerBlock;
     long long b = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
     TileB t{0, 0, 0, 0};
@@ -323,7 +421,7 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks)
 #pragma unroll
     for (int q = 0; q < kIpt; ++q) {
         const int k = lane + q * 32;
-        sidx[q] = (b < ntiles && k < t.ne) ? __ldg(t_src + t.e0 + k) : -1;
+        sidx[q] = (b < ntiles && k < t.ne) ? ld_stream(t_src + t.e0 + k, pol) : -1;
     }
     while (b < ntiles) {
         const long long bn = b + nw;
@@ -338,21 +436,33 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks)
 #pragma unroll
             for (int q = 0; q < kIpt; ++q) {
                 const int k = lane + q * 32;
-                sidx[q] = (bn < ntiles && k < tn.ne) ? __ldg(t_src + tn.e0 + k) : -1;
+                sidx[q] = (bn < ntiles && k < tn.ne) ? ld_stream(t_src + tn.e0 + k, pol) : -1;
             }
-            int re[kIpt];
+            if (t.nr == 0) {
+                // every item a link of one row that goes on: no merge
+                double sum = 0.0;
 #pragma unroll
-            for (int q = 0; q < kIpt; ++q) {
-                const int k = lane + q * 32;
-                re[q] = (k < t.nr) ? (int)(__ldg(t_ptr + t.r0 + 1 + k) - t.e0) : 0;
+                for (int q = 0; q < kIpt; ++q) {
+                    const int k = lane + q * 32;
+                    sum += (kHasW && k < t.ne) ? v[q] * (double)__ldg(t_w + t.e0 + k) : v[q];
+                }
+                sum = warp_sum(sum);
+                if (lane == 0) red_add(y + t.r0, sum);
+                b = bn;
+                t = tn;
+                continue;
             }
+            // (a tile seldom holds more than 32 rows)
+            int re = 0;
+            if (lane < t.nr) re = (int)(__ldg(t_ptr + t.r0 + 1 + lane) - t.e0);
             start0 = (int)(__ldg(t_ptr + t.r0) - t.e0);
 #pragma unroll
             for (int q = 0; q < kIpt; ++q) {
                 const int k = lane + q * 32;
                 if (k < t.ne) ws.val[k] = kHasW ? v[q] * (double)__ldg(t_w + t.e0 + k) : v[q];
-                if (k < t.nr) ws.end[k] = re[q];
             }
+            if (lane < t.nr) ws.end[lane] = re;
+            for (int k = lane + 32; k < t.nr; k += 32) ws.end[k] = (int)(__ldg(t_ptr + t.r0 + 1 + k) - t.e0);
         }
         if (lane == 0) ws.end[t.nr] = 0x7fffffff;
         __syncwarp();
@@ -361,7 +471,6 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks)
         long long rowA = -1, rowB = -1;
         double accA = 0.0, accB = 0.0;
         if (d < total) {
-            const int dend = min(d + kIpt, total);
             int lo = max(0, d - t.ne), hi = min(d, t.nr);
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
@@ -371,26 +480,28 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks)
             const int row_start = (i == 0) ? start0 : ws.end[i - 1];
             bool whole = (j == row_start);  // no in-link of row i before this lane
             double sum = 0.0;
-            int cnt = 0;
-            for (; d < dend; ++d) {
-                if (j < ws.end[i]) {
-                    sum += ws.val[j];
-                    ++j;
-                    ++cnt;
-                } else {
-                    if (!whole) {
+            int end = ws.end[i], j0 = j;  // the row's end; the lane's first in-link of the row
+#pragma unroll
+            for (int q = 0; q < kIpt; ++q) {
+                if (d + q < total) {
+                    const bool link = j < end;
+                    if (link) sum += ws.val[j];
+                    if (!link && whole && j > j0) red_add(y + (t.r0 + i), sum);
+                    if (!link && !whole) {
                         rowA = t.r0 + i;
                         accA = sum;
-                    } else if (cnt > 0) {
-                        red_add(y + (t.r0 + i), sum);
                     }
-                    sum = 0.0;
-                    cnt = 0;
-                    ++i;
-                    whole = true;
+                    if (!link) {
+                        sum = 0.0;
+                        j0 = j;
+                        ++i;
+                        end = ws.end[i];
+                        whole = true;
+                    }
+                    j += link ? 1 : 0;
                 }
             }
-            if (cnt > 0 || !whole) {
+            if (j > j0 || !whole) {
                 rowB = t.r0 + i;
                 accB = sum;
             }
@@ -423,7 +534,7 @@ __device__ __forceinline__ void power_publish(PowAcc<T>& acc, SweepSlot* sl, T* 
 }
 
 template <typename T, bool kHasW>
-__global__ void __launch_bounds__(kThreads, kPowerMinBlocks) k_power(SweepArgs<T> A) {
+__global__ void __launch_bounds__(kPowThreads, 1) k_power(SweepArgs<T> A) {
     DevState* st = A.st;
     SweepState* sw = A.sw;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
@@ -431,7 +542,8 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks) k_power(SweepArgs<T
         if (A.use_cond && lead) cudaGraphSetConditional(A.cond_loop, 0u);
         return;
     }
-    __shared__ PowWarp<T> sm[kWarpsPerBlock];
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    PowSmem<T>& sm = *reinterpret_cast<PowSmem<T>*>(dyn_smem);
     __shared__ T tscratch[4 * 32];
     __shared__ SweepCtl sc;
     __shared__ Control ctl;
@@ -478,7 +590,7 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks) k_power(SweepArgs<T
         for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
              i += (long long)gridDim.x * blockDim.x) {
             const T v = A.c[i];
-            A.mt[i] = v * __ldg(scale + i);
+            A.mt[source_of(A.rank, (int)i)] = v * __ldg(scale + i);
             A.facc[i] = T(0);
             acc.a += fabs(v);
             acc.s += v;
@@ -606,7 +718,8 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks) k_power(SweepArgs<T
         // ----------------------------------------------------------- move
         SweepSlot* nsl = &sw->slot[rot3(sc.p)];  // this move's sums and tile counter
         if (lead) sc.ts[0][0] = globaltimer();
-        power_tiles<T, kHasW>(A, mt_cur, mt_nxt, sm[threadIdx.x >> 5], &nsl->chunk_next, acc);
+        const int n_hot = load_hot<T>(A, mt_cur, sm);
+        power_tiles<T, kHasW>(A, mt_cur, mt_nxt, sm, n_hot, &nsl->chunk_next, acc);
         if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts[0] + 1 : nullptr))
             break;
         power_split_rows<T>(A, mt_nxt, acc);

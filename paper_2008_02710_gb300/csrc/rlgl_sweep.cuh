@@ -218,6 +218,8 @@ struct SweepArgs {
     Piece<T>* pieces;   // pieces of its long green rows
     int n_hubs;  // hub targets of the push, and the only one when there is one
     int hub1;
+    const int* rank;  // source order of mt and mt2 (see source_of)
+    const HotInfo* hot;  // its hot front
     T* mt;
     T* mt2;      // power sweep: the moved cash of every other move
     T* facc;     // power sweep: sums of rows split across tiles (zero at rest)
@@ -550,7 +552,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
         if (kPass == PASS_ALL || mv.dense) {
 #pragma unroll
             for (int q = 0; q < kV; ++q)
-                if (q * 32 < group && g + q * 32 < hi) A.mt[g + q * 32] = m[q];
+                if (q * 32 < group && g + q * 32 < hi) A.mt[source_of(A.rank, g + q * 32)] = m[q];
         }
         if constexpr (kPass == PASS_ALL) load(g0);
         if constexpr (kPass == PASS_SELECT) {
@@ -724,11 +726,11 @@ template <typename T>
 __device__ __forceinline__ void dense_from_lists(const SweepArgs<T>& A, SweepSmem<T>& sm) {
     int lo, hi, group;
     block_span<T>(A.n, lo, hi, group);
-    for (int i = lo + (int)threadIdx.x; i < hi; i += kSweepThreads) A.mt[i] = T(0);
+    for (int i = lo + (int)threadIdx.x; i < hi; i += kSweepThreads) A.mt[source_of(A.rank, i)] = T(0);
     __syncthreads();
     for (int k = threadIdx.x; k < sm.n_list; k += kSweepThreads) {
         const Green<T>* e = A.list + lo + k;
-        A.mt[__ldcg(&e->id)] = __ldcg(&e->m);
+        A.mt[source_of(A.rank, __ldcg(&e->id))] = __ldcg(&e->m);
     }
 }
 
