@@ -470,6 +470,11 @@ static SweepArgs<T> sweep_args(rlgl_ctx* ctx, const Conds& cd) {
     a.deg = ctx->deg;
     a.list = (Green<T>*)ctx->f_list;
     a.pieces = (Piece<T>*)ctx->pieces;
+    // Links and what a move reads or writes once a node leave the L2 first
+    // where the nodes' cash, 1/d and history take most of it (129 MB):
+    // symmetrised R-MAT 24 (268 MB), a move 294 -> 234 us; R-MAT 20 (17 MB),
+    // 31.1 -> 32.8 us, so not there.
+    a.beyond_l2 = ctx->n * (long long)(2 * sizeof(T) + 8) > (96ll << 20) ? 1 : 0;
     a.n_hubs = ctx->n_hubs;
     a.hub1 = ctx->hub1;
     a.col = ctx->col;

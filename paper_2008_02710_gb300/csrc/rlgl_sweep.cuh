@@ -22,9 +22,10 @@
 // and pushed in chunks of 1024 links: R-MAT 20, per-link threshold, a move
 // 34.5 -> 31.3 us (select 9.4 + 3.8 wait -> 8.4 + 2.3; push 20.4 -> 20.5, of
 // which 2.67 M scattered additions take about 18 however they are issued:
-// 23 us as a kernel of their own on the same links); symmetrised R-MAT 24,
-// a move 324 -> 268 us (select 158 -> 79, push 166 -> 189, see push_rows);
-// PageRank of an R-MAT graph of 500000 nodes 63 -> 48 us.
+// 23 us as a kernel of their own on the same links); PageRank of an R-MAT
+// graph of 500000 nodes 63 -> 48 us; symmetrised R-MAT 24, a move 317 -> 293
+// us, and 234 us with what a move touches once a node or link first to leave
+// L2 and no degree loaded beside 1/d (select 156 -> 78, push 161 -> 156).
 // With the stale threshold (Control::theta_lag) a move after the first of a
 // launch has no stats phase and no first barrier: its select gathers the
 // statistics of the cash it reads, and the next move's threshold and
@@ -216,6 +217,7 @@ struct SweepArgs {
     const int* deg;     // links of each row
     Green<T>* list;     // the sweep's green rows, each block's in its own part
     Piece<T>* pieces;   // pieces of its long green rows
+    int beyond_l2;  // the node arrays do not fit the L2 (see sweep_args)
     int n_hubs;  // hub targets of the push, and the only one when there is one
     int hub1;
     const int* rank;  // source order of mt and mt2 (see source_of)
@@ -293,6 +295,18 @@ __device__ __forceinline__ bool at_least(double v, double th) {
     const unsigned long long a = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
     return a >= (unsigned long long)__double_as_longlong(th) && a <= 0x7ff0000000000000ull;
 }
+
+// The out-degree of a node from its 1/d: FP32's 1/d is within 2^-24 of the
+// quotient and the reciprocal taken here within 2^-23, so that for d < 2^20
+// the result is within 2^-2 of d; beyond (and in FP64, where a division costs
+// more than the load) it is loaded. Beyond L2 the load is a sector a green
+// node.
+__device__ __forceinline__ int degree_of(float idg, const int* deg) {
+    float d;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(d) : "f"(idg));  // (within 2^-23)
+    return idg > 0x1p-20f ? __float2int_rn(d) : __ldg(deg);
+}
+__device__ __forceinline__ int degree_of(double, const int* deg) { return __ldg(deg); }
 
 // A block's hub targets (see kHubSlots) and their sums of the move.
 template <typename T>
@@ -409,15 +423,16 @@ __device__ __forceinline__ void add_edges(T* __restrict__ c, int (&j)[kU], const
 template <typename T, bool kHasW>
 __device__ __forceinline__ void push_row(const SweepArgs<T>& A, long long pos, int len, T m, HotSmem<T>& hot) {
     const int lane = threadIdx.x & 31;
+    const unsigned long long pol = stream_policy(A.beyond_l2);
     for (int o = 0; o < len; o += 128) {
         int j[4];
         T v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int e = o + q * 32 + lane;
-            j[q] = e < len ? __ldg(A.col + pos + e) : -1;
+            j[q] = e < len ? ld_run(A.col + pos + e, pol) : -1;
             v[q] = m;
-            if (kHasW && e < len) v[q] = m * (T)__ldg(A.w + pos + e);
+            if (kHasW && e < len) v[q] = m * (T)ld_run(A.w + pos + e, pol);
         }
         add_edges<T, 4>(A.c, j, v, A.n_hubs, A.hub1, hot);
     }
@@ -481,7 +496,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
             C[q] = idg[q] = T(0);
             if (q * 32 < group && i < hi) {
                 C[q] = __ldcg(A.c + i);
-                if (need_idg) idg[q] = __ldg(A.ideg + i);
+                if (need_idg) idg[q] = ld_stream(reinterpret_cast<const T*>(A.ideg) + i, stream_policy(A.beyond_l2));
             }
         }
     };
@@ -537,7 +552,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
             deg[q] = 0;
             if (gm >> q & 1u) {
                 m[q] = C[q] * (scale_is_idg ? idg[q] : __ldg(scale + i));
-                if (kPass == PASS_SELECT) deg[q] = __ldg(A.deg + i);
+                if (kPass == PASS_SELECT) deg[q] = need_idg ? degree_of(idg[q], A.deg + i) : __ldg(A.deg + i);
             }
         }
 #pragma unroll
@@ -547,7 +562,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
             acc.m += C[q];
             acc.ma += fabs(C[q]);
             A.c[i] = T(0);
-            red_add(A.H + i, widen(C[q]));  // no load: the L2 adds
+            red_add_stream(A.H + i, widen(C[q]), stream_policy(A.beyond_l2));  // no load: the L2 adds
         }
         if (kPass == PASS_ALL || mv.dense) {
 #pragma unroll
@@ -630,6 +645,7 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
         const T m = __ldcg(&A.pieces[p].m);
         push_row<T, kHasW>(A, pos, len, m, sm.hot);
     }
+    const unsigned long long pol = stream_policy(A.beyond_l2);
     const int nl = sm.n_list;
     const Green<T>* list;
     {
@@ -650,7 +666,7 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
             const int id = __ldcg(&e->id);
             m = __ldcg(&e->m);
             base = __ldg(A.row_ptr + id);
-            len = __ldg(A.deg + id);
+            len = (int)(__ldg(A.row_ptr + id + 1) - base);
             if (len > kHubRow) len = 0;  // in pieces
         }
         const unsigned int mid = __ballot_sync(0xffffffffu, len > kShortRow);
@@ -701,8 +717,8 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
                 const long long pos = __shfl_sync(0xffffffffu, base, k) + e;
                 v[q] = __shfl_sync(0xffffffffu, m, k);
                 if (e < E) {
-                    j[q] = __ldg(A.col + pos);
-                    if (kHasW) v[q] *= (T)__ldg(A.w + pos);
+                    j[q] = ld_run(A.col + pos, pol);
+                    if (kHasW) v[q] *= (T)ld_run(A.w + pos, pol);
                 }
             }
             add_edges<T, 4>(A.c, j, v, A.n_hubs, A.hub1, sm.hot);
