@@ -1395,17 +1395,17 @@ __global__ void __launch_bounds__(kThreads) k_push(
 // Returns this thread's scan value; s_key/s_val then hold every thread's
 // key and scan value.
 template <typename TV, int kBT = kThreads>
-__device__ __forceinline__ TV block_segscan(long long key, TV val, long long* s_key, TV* s_val) {
+__device__ __forceinline__ TV block_segscan(int key, TV val, int* s_key, TV* s_val) {
     constexpr int kW = kBT / 32;
     constexpr unsigned kWMask = kW >= 32 ? 0xffffffffu : ((1u << kW) - 1u);
-    __shared__ long long w_key[kW];
+    __shared__ int w_key[kW];
     __shared__ TV w_val[kW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     TV x = val;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         TV y = __shfl_up_sync(0xffffffffu, x, o);
-        long long ky = __shfl_up_sync(0xffffffffu, key, o);
+        int ky = __shfl_up_sync(0xffffffffu, key, o);
         if (lane >= o && ky == key) x += y;
     }
     if (lane == 31) {
@@ -1415,12 +1415,12 @@ __device__ __forceinline__ TV block_segscan(long long key, TV val, long long* s_
     __syncthreads();
     if (wid == 0 && lane < kW) {
         // the same scan over the warp tails
-        long long k = w_key[lane];
+        int k = w_key[lane];
         TV v = w_val[lane];
 #pragma unroll
         for (int o = 1; o < kW; o <<= 1) {
             TV y = __shfl_up_sync(kWMask, v, o);
-            long long ky = __shfl_up_sync(kWMask, k, o);
+            int ky = __shfl_up_sync(kWMask, k, o);
             if (lane >= o && ky == k) v += y;
         }
         w_val[lane] = v;
@@ -1452,7 +1452,7 @@ struct PullSmem {
     TV val[kBT * mp_ipt(kBT)];
     int end[kBT * mp_ipt(kBT) + 1];
     int start0;
-    long long ckey[kBT];
+    int ckey[kBT];
     TV cval[kBT];
 };
 
@@ -1474,6 +1474,7 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
                                            long long first, long long step, PullSmem<TV, kBT>& sm,
                                            unsigned long long* next = nullptr) {
     constexpr int kIpt = mp_ipt(kBT);  // merge items per thread: a tile is kBT * kIpt items
+    const unsigned long long pol = stream_policy();
     __shared__ long long s_tnext;
     long long b = first;
     if (next) {
@@ -1490,14 +1491,15 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
         {
             int sidx[kIpt];
             float wv[kIpt];
-            long long re[kIpt];
 #pragma unroll
             for (int q = 0; q < kIpt; ++q) {
                 const int k = threadIdx.x + q * kBT;
-                sidx[q] = (k < nedges) ? __ldg(t_src + e0 + k) : -1;
-                if (kHasW) wv[q] = (k < nedges) ? __ldg(t_w + e0 + k) : 0.0f;
-                re[q] = (k < nrows) ? __ldg(t_ptr + r0 + 1 + k) : 0;
+                sidx[q] = (k < nedges) ? ld_stream(t_src + e0 + k, pol) : -1;
+                if (kHasW) wv[q] = (k < nedges) ? ld_stream(t_w + e0 + k, pol) : 0.0f;
             }
+            // (a tile seldom holds more rows than the block has threads)
+            int re = 0;
+            if ((int)threadIdx.x < nrows) re = (int)(__ldg(t_ptr + r0 + 1 + threadIdx.x) - e0);
             TV v[kIpt];
 #pragma unroll
             for (int q = 0; q < kIpt; ++q) v[q] = (sidx[q] >= 0) ? ld_shared_data<kCg>(src + sidx[q]) : TV(0);
@@ -1505,8 +1507,9 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
             for (int q = 0; q < kIpt; ++q) {
                 const int k = threadIdx.x + q * kBT;
                 if (k < nedges) sm.val[k] = kHasW ? v[q] * (TV)wv[q] : v[q];
-                if (k < nrows) sm.end[k] = (int)(re[q] - e0);
             }
+            if ((int)threadIdx.x < nrows) sm.end[threadIdx.x] = re;
+            for (int k = threadIdx.x + kBT; k < nrows; k += kBT) sm.end[k] = (int)(__ldg(t_ptr + r0 + 1 + k) - e0);
         }
         if (threadIdx.x == 0) {
             sm.end[nrows] = 0x7fffffff;
@@ -1514,14 +1517,13 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
         }
         __syncthreads();
         const int total = nrows + nedges;
-        int d = threadIdx.x * kIpt;
-        const bool active = d < total;
+        const int d = threadIdx.x * kIpt;
         // head piece: the end of a row begun by earlier threads (rowA);
-        // tail piece: a row that continues past this thread (carry).
-        long long rowA = -1, rowB = -1;
+        // tail piece: a row that continues past this thread (carry). Rows
+        // are local to the tile.
+        int rowA = -1, rowB = -1;
         TV accA = TV(0), accB = TV(0);
-        if (active) {
-            const int dend = min(d + kIpt, total);
+        if (d < total) {
             int lo = max(0, d - nedges), hi = min(d, nrows);
             while (lo < hi) {
                 int mid = (lo + hi) >> 1;
@@ -1531,29 +1533,31 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
             const int row_start = (i == 0) ? sm.start0 : sm.end[i - 1];
             bool whole = (j == row_start);  // no edge of row i before this thread
             TV acc = TV(0);
-            int cnt = 0;
-            for (; d < dend; ++d) {
-                if (j < sm.end[i]) {
-                    acc += sm.val[j];
-                    ++j;
-                    ++cnt;
-                } else {
-                    if (!whole) {
-                        rowA = r0 + i;
+            int end = sm.end[i], j0 = j;    // the row's end; the thread's first edge of the row
+#pragma unroll
+            for (int q = 0; q < kIpt; ++q) {
+                if (d + q < total) {
+                    const bool link = j < end;
+                    if (link) acc += sm.val[j];
+                    if (!link && whole && j > j0) red_add(out + (r0 + i), (TO)acc);
+                    if (!link && !whole) {
+                        rowA = i;
                         accA = acc;
-                    } else if (cnt > 0) {
-                        red_add(out + (r0 + i), (TO)acc);
                     }
-                    acc = TV(0);
-                    cnt = 0;
-                    ++i;
-                    whole = true;
+                    if (!link) {
+                        acc = TV(0);
+                        j0 = j;
+                        ++i;
+                        end = sm.end[i];
+                        whole = true;
+                    }
+                    j += link ? 1 : 0;
                 }
             }
-            if (cnt > 0 || !whole) {
+            if (j > j0 || !whole) {
                 // the row continues past this thread (or began before it and
                 // has not ended here)
-                rowB = r0 + i;
+                rowB = i;
                 accB = acc;
             }
         }
@@ -1563,11 +1567,11 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
         if (rowA >= 0) {
             TV sum = accA;
             if (threadIdx.x > 0 && sm.ckey[threadIdx.x - 1] == rowA) sum += sm.cval[threadIdx.x - 1];
-            red_add(out + rowA, (TO)sum);
+            red_add(out + (r0 + rowA), (TO)sum);
         }
         // last active thread: its carry leaves the tile
         const int last = (total - 1) / kIpt;
-        if ((int)threadIdx.x == last && rowB >= 0) red_add(out + rowB, (TO)run);
+        if ((int)threadIdx.x == last && rowB >= 0) red_add(out + (r0 + rowB), (TO)run);
         __syncthreads();
         if (next) {
             b = s_tnext;
