@@ -664,8 +664,7 @@ static int power_grid(rlgl_ctx* ctx) {
     const int nb = ctx->prec == RLGL_MIXED ? power_fit<float>(ctx) : power_fit<double>(ctx);
     if (nb < 1) return 0;
     const long long fit = (long long)nb * ctx->sms;
-    // (a block's warps take three times its tiles' 2048 items at once)
-    long long want = (ctx->ntiles + 2) / 3;
+    long long want = ctx->ntiles;
     const long long nodes = (ctx->n + 4 * kPowThreads - 1) / (4 * kPowThreads);
     if (nodes > want) want = nodes;
     if (want < 1) want = 1;

@@ -74,8 +74,8 @@ constexpr int kPowThreads = 768;
 constexpr int kPowWarps = kPowThreads / 32;
 
 // Merge-path items per lane of a warp tile: 12 for FP32 cash (384-item
-// tiles), 8 for FP64 (256-item tiles, so that a block's static shared
-// memory stays within 48 KB).
+// tiles), 6 for FP64 (192-item tiles: what 24 warps' tiles take of the
+// shared memory is taken from L1).
 __host__ __device__ constexpr int power_ipt(int cash_bytes) { return cash_bytes == 4 ? 12 : 6; }
 
 // Shared memory of one warp of the power sweep: its merge-path tile (the
@@ -93,18 +93,19 @@ struct PowWarp {
 };
 
 // Hot sources kept in shared memory, and the block's dynamic shared memory.
-__host__ __device__ constexpr int hot_cap(int cash_bytes) { return cash_bytes == 4 ? 16384 : 4096; }
+__host__ __device__ constexpr int hot_cap(int cash_bytes) { return cash_bytes == 4 ? 14336 : 4096; }
 template <typename T>
 struct PowSmem {
     alignas(16) T hot[hot_cap((int)sizeof(T))];
     PowWarp<T> warp[kPowWarps];
 };
 
-// Per-thread sums of a move: ||C_{t+1}||_1, sum C_{t+1}, sum M_t, sum |M_t|
-// (in the cash type, combined per block and then in FP64).
+// Per-thread sums of a move: ||C_{t+1}||_1, sum C_{t+1} (in the cash type,
+// combined per block and then in FP64). Sum M_t and sum |M_t| are the same
+// two sums of the move before, for M_t = C_t.
 template <typename T>
 struct PowAcc {
-    T a, s, m, ma;
+    T a, s;
 };
 
 // Row epilogue of an all-green move: row r's in-link sum v is C_{t+1},r;
@@ -117,8 +118,6 @@ __device__ __forceinline__ void power_row_with(const SweepArgs<T>& A, T* __restr
     red_add(A.H + r, widen(old));  // M_t,r joins the history (no load: the L2 adds)
     acc.a += fabs(v);
     acc.s += v;
-    acc.m += old;
-    acc.ma += fabs(old);
 }
 
 template <typename T>
@@ -154,7 +153,11 @@ __device__ __forceinline__ T warp_segscan(K key, T val) {
     for (int o = 1; o < 32; o <<= 1) {
         const T y = __shfl_up_sync(0xffffffffu, val, o);
         const K ky = __shfl_up_sync(0xffffffffu, key, o);
-        if (lane >= o && ky == key) val += y;
+        const bool add = lane >= o && ky == key && key >= 0;
+        // (no run reaches this far, nor further; an FP64 addition holds the
+        // SM's FP64 pipe for 16 cycles)
+        if (sizeof(T) == 8 && !__any_sync(0xffffffffu, add)) break;
+        if (add) val += y;
     }
     return val;
 }
@@ -196,31 +199,29 @@ __device__ __forceinline__ void ld_over(double& v, const double* p, bool pred) {
 
 // One move's pull with the row epilogue, a warp per merge-path tile: the
 // warps of the grid take the tiles w, w + W, w + 2W, ... for all but the
-// last two rounds, and the rest one at a time from the counter `next` (lane
+// last two rounds (the first always), and the rest one at a time from the counter `next` (lane
 // 0 asks one turn ahead), so that warps end within about one tile of one
 // another. While a warp sums a tile, the next tile's bounds and in-link
 // sources are in flight. No block-wide barrier: a warp's lanes meet only at
 // __syncwarp. The pieces of rows that cross tile boundaries go into facc.
 template <typename T, bool kHasW>
 __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __restrict__ mt_cur,
-                                            T* __restrict__ mt_next, PowSmem<T>& sm, int n_hot,
+                                            PowSmem<T>& sm, int n_hot,
                                             unsigned long long* next, PowAcc<T>& acc) {
     constexpr int kPowIpt = power_ipt((int)sizeof(T));
     const int lane = threadIdx.x & 31;
     PowWarp<T>& ws = sm.warp[threadIdx.x >> 5];
     T* const rsum = ws.rsum();
     const unsigned long long pol = stream_policy();
-    // (tiles: at most 2^38 / 256, an int; rows: below 2^27)
+    // (tiles: at most 2^38 / 192, an int; rows: below 2^27)
     const int ntiles = (int)A.nwtiles;
     const int nw = (int)gridDim.x * kPowWarps;
-    const int w = (int)blockIdx.x * kPowWarps + (int)(threadIdx.x >> 5);
-    const int dyn0 = max(ntiles / nw - 2, 0) * nw;  // tiles below are taken in turn, the rest handed out
+    // (a warp's first tile: neighbours on different SMs, so that a small
+    // chain has its few tiles on all of them)
+    int b = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;
+    const int dyn0 = max(ntiles / nw - 2, 1) * nw;  // tiles below are taken in turn, the rest handed out
     const T* __restrict__ scale = row_scale(A.sf, A.s, T(0));
-    int b = w, grab = 0;
-    if (dyn0 == 0) {
-        if (lane == 0) b = (int)atomicAdd(next, 1ull);
-        b = __shfl_sync(0xffffffffu, b, 0);
-    }
+    int grab = 0;
     if (lane == 0 && b + nw >= dyn0) grab = (int)atomicAdd(next, 1ull);  // for the turn after
     TileB t{0, 0, 0, 0};
     int sidx[kPowIpt];
@@ -357,7 +358,9 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
         const int last = (total - 1) / kPowIpt;
         if (lane == last && rowB >= 0) atomicAdd(A.facc + t.r0 + rowB, run);
         __syncwarp();
-        // the rows that end in this tile and began in it
+        // the rows that end in this tile and began in it (the next move's
+        // buffer is taken here: held over the tile it would be a spill)
+        T* __restrict__ mt_next = mt_cur == A.mt ? A.mt2 : A.mt;
         for (int k = lane; k < t.nr; k += 32) {
             if (k == 0 && first_split) continue;
             if (k == lane)
@@ -521,16 +524,14 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks)
 // Block sums of the per-thread move sums into the slot (thread 0; FP64).
 template <typename T>
 __device__ __forceinline__ void power_publish(PowAcc<T>& acc, SweepSlot* sl, T* scratch) {
-    T v4[4] = {acc.a, acc.s, acc.m, acc.ma};
-    block_sum_n<T, 4>(v4, scratch);
+    T v4[2] = {acc.a, acc.s};
+    block_sum_n<T, 2>(v4, scratch);
     if (threadIdx.x == 0) {
         if (v4[0] != T(0)) atomicAdd(&sl->a, (double)v4[0]);
         if (v4[1] != T(0)) atomicAdd(&sl->s, (double)v4[1]);
-        if (v4[2] != T(0)) atomicAdd(&sl->msum, (double)v4[2]);
-        if (v4[3] != T(0)) atomicAdd(&sl->mabs, (double)v4[3]);
         if (blockIdx.x == 0) sl->tstamp = globaltimer();
     }
-    acc.a = acc.s = acc.m = acc.ma = T(0);
+    acc.a = acc.s = T(0);
 }
 
 template <typename T, bool kHasW>
@@ -574,13 +575,14 @@ __global__ void __launch_bounds__(kPowThreads, 1) k_power(SweepArgs<T> A) {
         sc.p = (int)(sw->bar.parity % 3u);  // the slot the first decision reads (clear)
         sc.want_refresh = 0;
         sc.have_lag = 0;
+        sc.mm = make_double2(0.0, 0.0);
     }
     __syncthreads();
     if (ctl.test_skip_barrier && blockIdx.x == gridDim.x - 1 && gridDim.x > 1) return;
-    // the moved cash of the current move (mt_cur) and of the next (mt_nxt)
+    // the moved cash of the current move; the next one's goes to the other
+    // of the two buffers
     T* mt_cur = A.mt;
-    T* mt_nxt = A.mt2;
-    PowAcc<T> acc{T(0), T(0), T(0), T(0)};
+    PowAcc<T> acc{T(0), T(0)};
 
     // ------------------------------------------------------- prologue
     // m~ = C s for the first move, the split rows' accumulators cleared, and
@@ -606,13 +608,13 @@ __global__ void __launch_bounds__(kPowThreads, 1) k_power(SweepArgs<T> A) {
             SweepSlot* sl = &sw->slot[sc.p];
             if (blockIdx.x == 0) clear_slot(&sw->slot[rot3(rot3(sc.p))]);  // read one decision ago
             const double2 as = ldcg_pair(&sl->a);         // ||C||_1 (and pr, unused)
-            const double2 mm = ldcg_pair(&sl->msum);      // the last move's sum M and sum |M|
             const double2 rts = ldcg_pair(&sl->reserve);  // block 0's timer in .y
             const double sum = __ldcg(&sl->s);
             const double l1 = as.x;
             const unsigned long long now = (unsigned long long)__double_as_longlong(rts.y);
-            sc.hsum += mm.x;
-            sc.habs += mm.y;
+            sc.hsum += sc.mm.x;  // the last move's sum M and sum |M|
+            sc.habs += sc.mm.y;
+            sc.mm = make_double2(sum, l1);  // and this move's, should it be made
             sc.l1 = l1;
             int stop = -1;
             bool skip = false, want_refresh = false;
@@ -719,10 +721,10 @@ __global__ void __launch_bounds__(kPowThreads, 1) k_power(SweepArgs<T> A) {
         SweepSlot* nsl = &sw->slot[rot3(sc.p)];  // this move's sums and tile counter
         if (lead) sc.ts[0][0] = globaltimer();
         const int n_hot = load_hot<T>(A, mt_cur, sm);
-        power_tiles<T, kHasW>(A, mt_cur, mt_nxt, sm, n_hot, &nsl->chunk_next, acc);
+        power_tiles<T, kHasW>(A, mt_cur, sm, n_hot, &nsl->chunk_next, acc);
         if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts[0] + 1 : nullptr))
             break;
-        power_split_rows<T>(A, mt_nxt, acc);
+        power_split_rows<T>(A, mt_cur == A.mt ? A.mt2 : A.mt, acc);
         power_publish<T>(acc, nsl, tscratch);
         if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts[0] + 3 : nullptr))
             break;
@@ -733,11 +735,7 @@ __global__ void __launch_bounds__(kPowThreads, 1) k_power(SweepArgs<T> A) {
             rec->phase_us[4] = (float)((sc.ts[0][1] - sc.ts[0][0]) + (sc.ts[0][3] - sc.ts[0][2])) * 1e-3f;
             rec->phase_us[5] = (float)((sc.ts[0][2] - sc.ts[0][1]) + (sc.ts[0][4] - sc.ts[0][3])) * 1e-3f;
         }
-        {
-            T* t = mt_cur;
-            mt_cur = mt_nxt;
-            mt_nxt = t;
-        }
+        mt_cur = mt_cur == A.mt ? A.mt2 : A.mt;
         if (threadIdx.x == 0) sc.p = rot3(sc.p);
         __syncthreads();
     }
