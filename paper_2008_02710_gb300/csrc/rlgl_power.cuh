@@ -42,6 +42,8 @@
 //   memory (half and a third of the gathers), merge steps without branches,
 //   one load of row ends a lane, no merge for tiles inside a row  85 / 2775
 //   and the links' loads not kept in L1 and first to leave L2     71 / 2557
+//   no register spilled, two sums a node instead of four          71 / 2295
+//   tiles from a counter of the block, not of the GPU             71 / 2136
 // (the start of the second row on its own machine, the rest beside it). More
 // hot sources are slower: what shared memory takes is taken from L1, which
 // the loads in flight need (36864: 170 / 6690 us with the same merge as the
@@ -74,9 +76,10 @@ constexpr int kPowThreads = 768;
 constexpr int kPowWarps = kPowThreads / 32;
 
 // Merge-path items per lane of a warp tile: 12 for FP32 cash (384-item
-// tiles), 6 for FP64 (192-item tiles: what 24 warps' tiles take of the
-// shared memory is taken from L1).
-__host__ __device__ constexpr int power_ipt(int cash_bytes) { return cash_bytes == 4 ? 12 : 6; }
+// tiles), 8 for FP64 (256-item tiles). A tile's joins and epilogue are FP64
+// additions, so that fewer items a tile cost more of them: 6 a lane, R-MAT of
+// 1.5 M nodes, 100 moves 14.8 -> 16.9 ms, of 20000 nodes 4.8 -> 5.25 ms.
+__host__ __device__ constexpr int power_ipt(int cash_bytes) { return cash_bytes == 4 ? 12 : 8; }
 
 // Shared memory of one warp of the power sweep: its merge-path tile (the
 // gathered in-link values, the row ends) and each row's in-link sum (local
@@ -98,6 +101,7 @@ template <typename T>
 struct PowSmem {
     alignas(16) T hot[hot_cap((int)sizeof(T))];
     PowWarp<T> warp[kPowWarps];
+    int next;  // the block's next tile to hand out
 };
 
 // Per-thread sums of a move: ||C_{t+1}||_1, sum C_{t+1} (in the cash type,
@@ -167,6 +171,7 @@ __device__ __forceinline__ T warp_segscan(K key, T val) {
 template <typename T>
 __device__ __forceinline__ int load_hot(const SweepArgs<T>& A, const T* __restrict__ mt, PowSmem<T>& sm) {
     const int n_hot = A.hot ? __ldg(&A.hot->count) : 0;
+    if (threadIdx.x == 0) sm.next = kPowWarps;  // (every warp's first is its own)
     constexpr int kPer = 16 / (int)sizeof(T);
     const int nv = n_hot / kPer;
     const float4* src = reinterpret_cast<const float4*>(mt);
@@ -197,32 +202,29 @@ __device__ __forceinline__ void ld_over(double& v, const double* p, bool pred) {
                  : "l"(p), "r"((int)pred));
 }
 
-// One move's pull with the row epilogue, a warp per merge-path tile: the
-// warps of the grid take the tiles w, w + W, w + 2W, ... for all but the
-// last two rounds (the first always), and the rest one at a time from the counter `next` (lane
-// 0 asks one turn ahead), so that warps end within about one tile of one
-// another. While a warp sums a tile, the next tile's bounds and in-link
+// One move's pull with the row epilogue, a warp per merge-path tile: block k
+// of G takes the tiles k, k + G, k + 2G, ..., its warps one after another
+// from a counter in shared memory (lane 0 asks one turn ahead). Tiles are of
+// one size, so that the blocks end together. With the last two rounds handed
+// out one at a time from a counter of the whole GPU, which 3648 warps asked:
+// symmetrised R-MAT 24, 60 moves, 137.7 ms against 128.1; weighted R-MAT of
+// 2 M nodes, 20 moves, 4.06 against 3.89; R-MAT 20 4.32 against 4.34. While a warp sums a tile, the next tile's bounds and in-link
 // sources are in flight. No block-wide barrier: a warp's lanes meet only at
 // __syncwarp. The pieces of rows that cross tile boundaries go into facc.
 template <typename T, bool kHasW>
 __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __restrict__ mt_cur,
-                                            PowSmem<T>& sm, int n_hot,
-                                            unsigned long long* next, PowAcc<T>& acc) {
+                                            PowSmem<T>& sm, int n_hot, PowAcc<T>& acc) {
     constexpr int kPowIpt = power_ipt((int)sizeof(T));
     const int lane = threadIdx.x & 31;
     PowWarp<T>& ws = sm.warp[threadIdx.x >> 5];
     T* const rsum = ws.rsum();
     const unsigned long long pol = stream_policy();
-    // (tiles: at most 2^38 / 192, an int; rows: below 2^27)
+    // (tiles: at most 2^38 / 256, an int; rows: below 2^27)
     const int ntiles = (int)A.nwtiles;
-    const int nw = (int)gridDim.x * kPowWarps;
-    // (a warp's first tile: neighbours on different SMs, so that a small
-    // chain has its few tiles on all of them)
     int b = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;
-    const int dyn0 = max(ntiles / nw - 2, 1) * nw;  // tiles below are taken in turn, the rest handed out
     const T* __restrict__ scale = row_scale(A.sf, A.s, T(0));
     int grab = 0;
-    if (lane == 0 && b + nw >= dyn0) grab = (int)atomicAdd(next, 1ull);  // for the turn after
+    if (lane == 0) grab = atomicAdd(&sm.next, 1);  // for the turn after
     TileB t{0, 0, 0, 0};
     int sidx[kPowIpt];
     if (b < ntiles) t = tile_bounds(A.wtile_r, A.wtile_e, b);
@@ -253,9 +255,8 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
                 if (kHasW && k < t.ne) asm volatile("prefetch.global.L1 [%0];" ::"l"(A.t_w + t.e0 + k));
             }
             // the next tile's bounds and sources, in flight over this tile
-            bn = b + nw;
-            if (bn >= dyn0) bn = dyn0 + __shfl_sync(0xffffffffu, grab, 0);
-            if (bn < ntiles && bn + nw >= dyn0 && lane == 0) grab = (int)atomicAdd(next, 1ull);
+            bn = __shfl_sync(0xffffffffu, grab, 0) * (int)gridDim.x + (int)blockIdx.x;
+            if (bn < ntiles && lane == 0) grab = atomicAdd(&sm.next, 1);
             if (bn < ntiles) tn = tile_bounds(A.wtile_r, A.wtile_e, bn);
 #pragma unroll
             for (int q = 0; q < kPowIpt; ++q) {
@@ -718,10 +719,10 @@ __global__ void __launch_bounds__(kPowThreads, 1) k_power(SweepArgs<T> A) {
         if (sc.leave) return;
 
         // ----------------------------------------------------------- move
-        SweepSlot* nsl = &sw->slot[rot3(sc.p)];  // this move's sums and tile counter
+        SweepSlot* nsl = &sw->slot[rot3(sc.p)];  // this move's sums
         if (lead) sc.ts[0][0] = globaltimer();
         const int n_hot = load_hot<T>(A, mt_cur, sm);
-        power_tiles<T, kHasW>(A, mt_cur, sm, n_hot, &nsl->chunk_next, acc);
+        power_tiles<T, kHasW>(A, mt_cur, sm, n_hot, acc);
         if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns, blockIdx.x == 0 ? sc.ts[0] + 1 : nullptr))
             break;
         power_split_rows<T>(A, mt_cur == A.mt ? A.mt2 : A.mt, acc);
