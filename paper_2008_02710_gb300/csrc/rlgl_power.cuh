@@ -525,16 +525,27 @@ __global__ void __launch_bounds__(kThreads, kPowerMinBlocks)
     }
 }
 
-// Block sums of the per-thread move sums into the slot (thread 0; FP64).
+// Block sums of the per-thread move sums into the slot: in the cash type up
+// to three warps, in FP64 beyond (a block holds 24).
 template <typename T>
-__device__ __forceinline__ void power_publish(PowAcc<T>& acc, SweepSlot* sl, T* scratch) {
-    T v4[2] = {acc.a, acc.s};
-    block_sum_n<T, 2>(v4, scratch);
-    if (threadIdx.x == 0) {
-        if (v4[0] != T(0)) atomicAdd(&sl->a, (double)v4[0]);
-        if (v4[1] != T(0)) atomicAdd(&sl->s, (double)v4[1]);
-        if (blockIdx.x == 0) sl->tstamp = globaltimer();
+__device__ __forceinline__ void power_publish(PowAcc<T>& acc, SweepSlot* sl, T (&scratch)[2][kPowWarps]) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const T a = warp_sum(acc.a), s = warp_sum(acc.s);
+    if (lane == 0) {
+        scratch[0][wid] = a;
+        scratch[1][wid] = s;
     }
+    __syncthreads();
+    if (wid < 2) {
+        T v = lane < kPowWarps ? scratch[wid][lane] : T(0);
+        v += __shfl_down_sync(0xffffffffu, v, 16);
+        v += __shfl_down_sync(0xffffffffu, v, 8);
+        double x = v;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        if (lane == 0 && x != 0.0) atomicAdd(wid == 0 ? &sl->a : &sl->s, x);
+    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) sl->tstamp = globaltimer();
     acc.a = acc.s = T(0);
 }
 
@@ -549,7 +560,7 @@ __global__ void __launch_bounds__(kPowThreads, 1) k_power(SweepArgs<T> A) {
     }
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     PowSmem<T>& sm = *reinterpret_cast<PowSmem<T>*>(dyn_smem);
-    __shared__ T tscratch[4 * 32];
+    __shared__ T tscratch[2][kPowWarps];
     __shared__ SweepCtl sc;
     __shared__ Control ctl;
     __shared__ double s_l1_refresh;

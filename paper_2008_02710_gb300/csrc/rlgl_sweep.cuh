@@ -474,9 +474,15 @@ __device__ __forceinline__ void block_span(int n, int& lo, int& hi, int& group) 
 // in mt, no list).
 enum Pass : int { PASS_STATS, PASS_SELECT, PASS_ALL };
 
-// The block's warps take its groups of nodes one after another from a
+// With FP32 cash, and for the statistics, warp w of a block takes its groups
+// of nodes w, w + 32, ..., so that one cash has one sum, and one threshold
+// from it, in every run. (From a counter, as the warps became free, sum v of
+// the same cash differed by up to 1e-8 of itself from run to run, and with it
+// two or three of symmetrised R-MAT 24's green nodes.) An FP64 selection,
+// whose sums differ by 1e-16 whatever their order, takes its groups from a
 // counter in shared memory (zero at the start of a pass; warp w starts with
-// group w); the next group's cash is loaded before the current one is listed.
+// group w): weighted R-MAT 22, 12 moves, 2788 -> 2766 us. The next group's
+// cash is loaded before the current one is listed.
 template <typename T, bool kHasW, int kPass>
 __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<T>& mv, const SchedAux& ax,
                                           SweepSmem<T>& sm, NodeAcc<T>& acc) {
@@ -504,9 +510,13 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
     load(g0);
     while (g0 < hi) {
         const int g = g0 + lane;
-        int nxt = 0;
-        if (lane == 0) nxt = atomicAdd(&sm.next_group, 1);
-        g0 = lo + (kSweepWarps + __shfl_sync(0xffffffffu, nxt, 0)) * group;
+        if constexpr (kPass == PASS_STATS || sizeof(T) == 4) {
+            g0 += kSweepWarps * group;
+        } else {
+            int nxt = 0;
+            if (lane == 0) nxt = atomicAdd(&sm.next_group, 1);
+            g0 = lo + (kSweepWarps + __shfl_sync(0xffffffffu, nxt, 0)) * group;
+        }
         unsigned int gm = 0u;  // green nodes of this lane
 #pragma unroll
         for (int q = 0; q < kV; ++q) {
@@ -951,26 +961,28 @@ __device__ __forceinline__ int rot3(int q) { return q == 2 ? 0 : q + 1; }
 // Sums of four values a lane over the warp: the total of v[k] ends in lanes
 // 8 k to 8 k + 7. Six additions in a row of five steps, where four sums one
 // by one take twenty (an FP64 addition holds the SM's FP64 pipe for 16
-// cycles).
-template <typename T>
-__device__ __forceinline__ T warp_sum4(const T (&v)[4]) {
+// cycles). The first two steps are in T, the last three (eight partial sums)
+// in R.
+template <typename R, typename T>
+__device__ __forceinline__ R warp_sum4(const T (&v)[4]) {
     const int lane = threadIdx.x & 31;
     const bool hi = (lane & 16) != 0, hh = (lane & 8) != 0;
     T a = hi ? v[2] : v[0], b = hi ? v[3] : v[1];
     a += __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
     b += __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 16);
-    T x = hh ? b : a;
-    x += __shfl_xor_sync(0xffffffffu, hh ? a : b, 8);
+    T half = hh ? b : a;
+    half += __shfl_xor_sync(0xffffffffu, hh ? a : b, 8);
+    R x = half;
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
 }
 
 // The block's sums of a pass into the move's slot: sum m, sum |m|, ||C||_1,
-// sum v^r in the cash type, the links and green nodes packed (green: the
-// block's count of them, NULL for none); one FP64 (or
-// 64-bit) addition per total that is not zero. A grid barrier follows every
-// call, so the scratch is free again.
+// sum v^r in the cash type up to four warps, in FP64 beyond, the links and
+// green nodes packed (green: the block's count of them, NULL for none); one
+// FP64 (or 64-bit) addition per total that is not zero. A grid barrier
+// follows every call, so the scratch is free again.
 template <typename T>
 struct PubSmem {
     T v[4][kSweepWarps];
@@ -982,7 +994,7 @@ __device__ __forceinline__ void publish(const NodeAcc<T>& acc, SweepSlot* sl, Pu
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     {
         const T v[4] = {acc.m, acc.ma, acc.a, acc.pr};
-        const T x = warp_sum4(v);
+        const T x = warp_sum4<T>(v);
         const unsigned long long r = warp_sum(acc.edges);
         if ((lane & 7) == 0) ps.v[lane >> 3][wid] = x;
         if (lane == 0) ps.r[wid] = r;
@@ -990,9 +1002,9 @@ __device__ __forceinline__ void publish(const NodeAcc<T>& acc, SweepSlot* sl, Pu
     __syncthreads();
     if (wid == 0) {
         const T v[4] = {ps.v[0][lane], ps.v[1][lane], ps.v[2][lane], ps.v[3][lane]};
-        const T x = warp_sum4(v);
+        const double x = warp_sum4<double>(v);
         double* out = lane < 8 ? &sl->msum : (lane < 16 ? &sl->mabs : (lane < 24 ? &sl->a : &sl->pr));
-        if ((lane & 7) == 0 && x != T(0)) atomicAdd(out, (double)x);
+        if ((lane & 7) == 0 && x != 0.0) atomicAdd(out, x);
         if (lane == 0 && blockIdx.x == 0 && stamp) sl->tstamp = globaltimer();
     } else if (wid == 1) {
         const unsigned long long r = (warp_sum(ps.r[lane]) << kCountBits) + (green ? (unsigned int)*green : 0u);
