@@ -3,7 +3,7 @@
 // costs three grid barriers (two with the stale threshold) instead of three
 // to four kernel launches, their drain and their serial last-block tails.
 //
-// One block of 1024 threads an SM owns a contiguous span of the nodes; a move is
+// One block of 1024 threads an SM owns every G-th group of nodes; a move is
 //   stats   : the statistics of its nodes' cash; block sums go to one FP64
 //             atomic per statistic in the move's slot;
 //   barrier ; every block reads the totals and takes the same decisions
@@ -260,7 +260,7 @@ __device__ __noinline__ T pow_r(T x, int r) {
 
 // ------------------------------------------------------- the node passes
 //
-// A block owns a contiguous span of nodes and selects, lists and pushes its
+// A block owns its groups of nodes (OwnNodes) and selects, lists and pushes its
 // own green rows; only rows of more than kHubRow links are cut into pieces
 // that all blocks share. So a row's entry is written and read on the same SM,
 // no space has to be reserved across the GPU, and nothing of a red node is
@@ -454,19 +454,35 @@ __device__ __forceinline__ void flush_hubs(const SweepArgs<T>& A, HotSmem<T>& ho
         }
 }
 
-// The nodes [lo, hi) of this block: one contiguous span per block, a
-// multiple of 32 nodes, and the nodes its warps take at a time: 128 where
-// every warp gets several such groups, down to 32 where they would not
-// otherwise all get one.
+// The nodes of a block: every gridDim.x-th group of consecutive nodes, from
+// group blockIdx.x on, so that nodes near one another (the green range of a
+// block-round-robin move, a host's pages, the long rows of ids sorted by
+// degree) fall to all blocks alike. A group is what a warp takes at a time:
+// 128 nodes where every warp gets several of them, down to 32 where they
+// would not otherwise all get one.
+// Measured against one contiguous span a block, R-MAT 20, 40 moves of eight
+// blocks in turn: 3562 -> 1858 us, FP64 3782 -> 1994; ids sorted by degree,
+// per-link threshold, 60 moves: 11476 -> 7705 us, FP64 10717 -> 6609; ids at
+// random: 2699 -> 2706 us, FP64 3298 -> 3268.
 template <typename T>
-__device__ __forceinline__ void block_span(int n, int& lo, int& hi, int& group) {
-    const int nb = (int)gridDim.x;
-    const int span = (int)(((long long)n + nb * 32ll - 1) / (nb * 32ll)) * 32;
-    lo = (int)min((long long)blockIdx.x * span, (long long)n);
-    hi = (int)min((long long)lo + span, (long long)n);
-    group = span >= 128 * 2 * kSweepWarps ? 128 : (span >= 64 * kSweepWarps ? 64 : 32);
-    if (group > 32 * NodeVec<T>::kV) group = 32 * NodeVec<T>::kV;
-}
+struct OwnNodes {
+    int shift;  // log2 of a group's nodes
+    __device__ __forceinline__ explicit OwnNodes(int n) {
+        const int mean = (n + (int)gridDim.x - 1) / (int)gridDim.x;  // nodes a block
+        shift = mean >= 128 * 2 * kSweepWarps ? 7 : (mean >= 64 * kSweepWarps ? 6 : 5);
+        static_assert(NodeVec<T>::kV == 2 || NodeVec<T>::kV == 4, "a group is at most 64 or 128 nodes");
+        if (NodeVec<T>::kV == 2 && shift > 6) shift = 6;
+    }
+    __device__ __forceinline__ int group() const { return 1 << shift; }
+    // The first node of the block's group j (n or more: it has no such
+    // group). (n < 2^27, and a warp asks for one group beyond the block's last
+    // at most: below 2^31)
+    __device__ __forceinline__ int first(int j) const { return (j * (int)gridDim.x + (int)blockIdx.x) << shift; }
+    // The block's node k, counted over its groups. Only the chain's last
+    // group may hold fewer nodes, and it is the last of its block: of a block
+    // with m nodes, nodes 0 to m - 1 are in range.
+    __device__ __forceinline__ int node(int k) const { return first(k >> shift) + (k & ((1 << shift) - 1)); }
+};
 
 // The passes over the nodes. STATS: the statistics of the cash. SELECT: the
 // green nodes give up their cash (m_i = C_i, C_i <- 0, H_i += m_i) and are
@@ -488,8 +504,8 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
                                           SweepSmem<T>& sm, NodeAcc<T>& acc) {
     constexpr int kV = NodeVec<T>::kV;
     const int lane = threadIdx.x & 31;
-    int lo, hi, group;
-    block_span<T>(A.n, lo, hi, group);
+    const OwnNodes<T> own(A.n);
+    const int n = A.n, group = own.group();
     const bool need_idg = mv.link && (kPass == PASS_STATS || mv.acc || mv.sched == SCHED_LINK);
     const bool scale_is_idg = !kHasW && need_idg;  // unit weights: s_i = 1/d_i
     const T* scale = row_scale(A.sf, A.s, T(0));
@@ -500,28 +516,28 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
         for (int q = 0; q < kV; ++q) {
             const int i = g + q * 32 + lane;
             C[q] = idg[q] = T(0);
-            if (q * 32 < group && i < hi) {
+            if (q * 32 < group && i < n) {
                 C[q] = __ldcg(A.c + i);
                 if (need_idg) idg[q] = ld_stream(reinterpret_cast<const T*>(A.ideg) + i, stream_policy(A.beyond_l2));
             }
         }
     };
-    int g0 = lo + (int)(threadIdx.x >> 5) * group;
+    int g0 = own.first((int)(threadIdx.x >> 5));
     load(g0);
-    while (g0 < hi) {
+    while (g0 < n) {
         const int g = g0 + lane;
         if constexpr (kPass == PASS_STATS || sizeof(T) == 4) {
-            g0 += kSweepWarps * group;
+            g0 += (int)gridDim.x * kSweepWarps << own.shift;
         } else {
             int nxt = 0;
             if (lane == 0) nxt = atomicAdd(&sm.next_group, 1);
-            g0 = lo + (kSweepWarps + __shfl_sync(0xffffffffu, nxt, 0)) * group;
+            g0 = own.first(kSweepWarps + __shfl_sync(0xffffffffu, nxt, 0));
         }
         unsigned int gm = 0u;  // green nodes of this lane
 #pragma unroll
         for (int q = 0; q < kV; ++q) {
             const int i = g + q * 32;
-            if (q * 32 >= group || i >= hi) continue;
+            if (q * 32 >= group || i >= n) continue;
             const T av = fabs(C[q]);
             const T tv = mv.link ? av * idg[q] : av;
             if (kPass == PASS_STATS || mv.acc) {
@@ -551,7 +567,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
                 k += __popc(__ballot_sync(0xffffffffu, (gm >> q & 1u) != 0u));
             }
             if (lane == 0 && k > 0) k = atomicAdd(&sm.n_list, k);
-            k = lo + __shfl_sync(0xffffffffu, k, 0);
+            k = __shfl_sync(0xffffffffu, k, 0);
         }
         T m[kV];  // moved cash per weight
         int deg[kV];
@@ -577,7 +593,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
         if (kPass == PASS_ALL || mv.dense) {
 #pragma unroll
             for (int q = 0; q < kV; ++q)
-                if (q * 32 < group && g + q * 32 < hi) A.mt[source_of(A.rank, g + q * 32)] = m[q];
+                if (q * 32 < group && g + q * 32 < n) A.mt[source_of(A.rank, g + q * 32)] = m[q];
         }
         if constexpr (kPass == PASS_ALL) load(g0);
         if constexpr (kPass == PASS_SELECT) {
@@ -589,7 +605,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
                     Green<T> e;
                     e.id = g + q * 32;
                     e.m = m[q];
-                    A.list[k + __popc(bal & ((1u << lane) - 1u))] = e;
+                    A.list[own.node(k + __popc(bal & ((1u << lane) - 1u)))] = e;
                 }
                 k += __popc(bal);
                 acc.edges += (unsigned int)deg[q];
@@ -624,13 +640,15 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
     }
 }
 
-// A thread's share of sum v^r over the nodes [lo, hi) for r > 2 (ideg: 1/d
+// A thread's share of sum v^r over the block's nodes for r > 2 (ideg: 1/d
 // for the per-link v, else NULL), out of line: rare, and a call to pow inside
 // the node passes would cost them registers.
 template <typename T>
-__device__ __noinline__ T pow_sum(const T* c, const T* ideg, int lo, int hi, int r) {
+__device__ __noinline__ T pow_sum(const T* c, const T* ideg, int n, int r) {
     T sum = T(0);
-    for (int i = lo + (int)threadIdx.x; i < hi; i += kSweepThreads) {
+    const OwnNodes<T> own(n);
+    for (int k = threadIdx.x; own.node(k) < n; k += kSweepThreads) {
+        const int i = own.node(k);
         const T av = fabs(__ldcg(c + i));
         sum += (T)pow(ideg ? av * __ldg(ideg + i) : av, (T)r);
     }
@@ -657,12 +675,7 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
     }
     const unsigned long long pol = stream_policy(A.beyond_l2);
     const int nl = sm.n_list;
-    const Green<T>* list;
-    {
-        int lo, hi, group;
-        block_span<T>(A.n, lo, hi, group);
-        list = A.list + lo;
-    }
+    const OwnNodes<T> own(A.n);
     for (;;) {
         int z = 0;
         if (lane == 0) z = atomicAdd(&sm.next_list, 32);
@@ -672,7 +685,7 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
         long long base = 0;
         T m = T(0);
         if (z + lane < nl) {
-            const Green<T>* e = list + z + lane;
+            const Green<T>* e = A.list + own.node(z + lane);
             const int id = __ldcg(&e->id);
             m = __ldcg(&e->m);
             base = __ldg(A.row_ptr + id);
@@ -747,15 +760,14 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
 
 // The dense moved cash of a move that pulls though it was not expected to:
 // cleared (PASS 0), then set from the block's lists (after a barrier: other
-// blocks' spans do not matter, but the pull reads all of them).
+// blocks' nodes do not matter, but the pull reads all of them).
 template <typename T>
 __device__ __forceinline__ void dense_from_lists(const SweepArgs<T>& A, SweepSmem<T>& sm) {
-    int lo, hi, group;
-    block_span<T>(A.n, lo, hi, group);
-    for (int i = lo + (int)threadIdx.x; i < hi; i += kSweepThreads) A.mt[source_of(A.rank, i)] = T(0);
+    const OwnNodes<T> own(A.n);
+    for (int k = threadIdx.x; own.node(k) < A.n; k += kSweepThreads) A.mt[source_of(A.rank, own.node(k))] = T(0);
     __syncthreads();
     for (int k = threadIdx.x; k < sm.n_list; k += kSweepThreads) {
-        const Green<T>* e = A.list + lo + k;
+        const Green<T>* e = A.list + own.node(k);
         A.mt[source_of(A.rank, __ldcg(&e->id))] = __ldcg(&e->m);
     }
 }
@@ -1014,10 +1026,8 @@ __device__ __forceinline__ void publish(const NodeAcc<T>& acc, SweepSlot* sl, Pu
 
 template <typename T, bool kHasW>
 __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
-    DevState* st = A.st;
-    SweepState* sw = A.sw;
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
-    if (st->done) {
+    if (A.st->done) {
         if (A.use_cond && lead) cudaGraphSetConditional(A.cond_loop, 0u);
         return;
     }
@@ -1032,7 +1042,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
     __shared__ double s_l1_refresh;
     __shared__ unsigned long long s_limit_ns;  // the solve's time limit
     {
-        const unsigned int* src = reinterpret_cast<const unsigned int*>(&st->ctl);
+        const unsigned int* src = reinterpret_cast<const unsigned int*>(&A.st->ctl);
         unsigned int* dst = reinterpret_cast<unsigned int*>(&ctl);
         for (int k = threadIdx.x; k < (int)(sizeof(Control) / 4); k += blockDim.x) dst[k] = src[k];
         for (int k = threadIdx.x; k < kHubSlots; k += blockDim.x) {
@@ -1044,31 +1054,31 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
     __syncthreads();
     const int n = A.n;
     if (threadIdx.x == 0) {
-        s_l1_refresh = st->l1_refresh;
+        s_l1_refresh = A.st->l1_refresh;
         // an integer number of ns exceeds the limit when it exceeds its floor
         s_limit_ns = ctl.time_limit_ns < 9e18 ? (unsigned long long)ctl.time_limit_ns : ~0ull;
-        sc.moves = st->moves;
-        sc.solve_moves = st->solve_moves;
-        sc.iters = st->iters;
-        sc.mask_cursor = st->mask_cursor;
-        sc.tot_green = st->tot_green;
-        sc.tot_edges = st->tot_edges;
-        sc.push_moves = st->push_moves;
-        sc.pull_moves = st->pull_moves;
-        sc.edges = st->edges;  // the last move's (0 at the start of a solve)
-        sc.hsum = st->hsum;
-        sc.habs = st->habs;
-        sc.t_start = st->t_start;
-        sc.fresh = st->fresh;
-        sc.stall_mark = st->stall_mark;
-        sc.stall_count = st->stall_count;
+        sc.moves = A.st->moves;
+        sc.solve_moves = A.st->solve_moves;
+        sc.iters = A.st->iters;
+        sc.mask_cursor = A.st->mask_cursor;
+        sc.tot_green = A.st->tot_green;
+        sc.tot_edges = A.st->tot_edges;
+        sc.push_moves = A.st->push_moves;
+        sc.pull_moves = A.st->pull_moves;
+        sc.edges = A.st->edges;  // the last move's (0 at the start of a solve)
+        sc.hsum = A.st->hsum;
+        sc.habs = A.st->habs;
+        sc.t_start = A.st->t_start;
+        sc.fresh = A.st->fresh;
+        sc.stall_mark = A.st->stall_mark;
+        sc.stall_count = A.st->stall_count;
         // Every barrier adds exactly the grid size, and no barrier can
         // complete before this block arrives: rounding down what has arrived
         // gives the count at the start of this launch.
-        const unsigned long long arr = ld_acquire_u64(&sw->bar.arrived);
+        const unsigned long long arr = ld_acquire_u64(&A.sw->bar.arrived);
         sc.target = arr - arr % gridDim.x;
-        sc.p = (int)(sw->bar.parity % 3u);
-        sc.tk_pass = sw->bar.tk_pass;
+        sc.p = (int)(A.sw->bar.parity % 3u);
+        sc.tk_pass = A.sw->bar.tk_pass;
         sc.limit = ctl.pull_crossover * (double)ctl.nnz;
         sc.l1 = sc.sumr = sc.mean = 0.0;
         sc.have_lag = sc.leave = sc.made = sc.owed = sc.want_refresh = sc.tb = 0;
@@ -1088,13 +1098,11 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
     if (ctl.test_skip_barrier && blockIdx.x == gridDim.x - 1 && gridDim.x > 1) return;
 
     auto pow_share = [&]() {
-        int lo, hi, group;
-        block_span<T>(n, lo, hi, group);
-        return pow_sum<T>(A.c, mv.link ? A.ideg : nullptr, lo, hi, mv.r);
+        return pow_sum<T>(A.c, mv.link ? A.ideg : nullptr, n, mv.r);
     };
     // Block 0's duties of the last move, while it waits at a barrier.
     auto owed = [&]() {
-        if (blockIdx.x == 0) write_owed(sc, st, A.log);
+        if (blockIdx.x == 0) write_owed(sc, A.st, A.log);
     };
     // The end of a move (thread 0, while its block waits at the move's last
     // barrier): the stop test and the re-derivation triggers of the stale
@@ -1179,10 +1187,10 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
                 NodeAcc<T> acc = kNoAcc<T>;
                 node_pass<T, kHasW, PASS_STATS>(A, mv, sc.ax, sm, acc);
                 if (mv.r > 2) acc.pr = pow_share();
-                publish<T>(acc, &sw->slot[sc.p], ps, true);
+                publish<T>(acc, &A.sw->slot[sc.p], ps, true);
             }
             auto control = [&]() {
-                const SweepSlot* sl = &sw->slot[sc.p];
+                const SweepSlot* sl = &A.sw->slot[sc.p];
                 const double2 apr = ldcg_pair(&sl->a);
                 const double2 rts = ldcg_pair(&sl->reserve);
                 const double l1 = apr.x;
@@ -1191,7 +1199,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
                 if (threadIdx.x != 0) return;
                 // (every block is done with the last move's slot; a launch
                 // that ends here has no move that would clear it)
-                if (blockIdx.x == 0) clear_slot(&sw->slot[rot3(rot3(sc.p))]);
+                if (blockIdx.x == 0) clear_slot(&A.sw->slot[rot3(rot3(sc.p))]);
                 sc.l1 = l1;
                 sc.sumr = sumr;
                 sc.mean = q.y;
@@ -1226,7 +1234,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
                 }
                 set_move<T>(sc, ctl, mv, sm, A.masks, n, l1, q.y);
             };
-            if (!grid_barrier_with(&sw->bar, sc.target, ctl.barrier_limit_ns,
+            if (!grid_barrier_with(&A.sw->bar, sc.target, ctl.barrier_limit_ns,
                                    blockIdx.x == 0 ? sc.ts[sc.tb] + 1 : nullptr, owed, control))
                 goto aborted;
         }
@@ -1249,13 +1257,13 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
                 const int width = hi >= kRadixBits ? kRadixBits : hi;
                 const int shift = hi - width;
                 const unsigned int q = sc.tk_pass;
-                sweep_radix_count<T>(A.c, n, sw->tk_hist[q % 3u], sc.tk_prefix, shift, width, sm.hist);
-                if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns)) goto aborted;
+                sweep_radix_count<T>(A.c, n, A.sw->tk_hist[q % 3u], sc.tk_prefix, shift, width, sm.hist);
+                if (!grid_barrier(&A.sw->bar, sc.target, ctl.barrier_limit_ns)) goto aborted;
                 if (blockIdx.x == 0) {
-                    unsigned int* old = sw->tk_hist[(q + 2u) % 3u];
+                    unsigned int* old = A.sw->tk_hist[(q + 2u) % 3u];
                     for (int b = threadIdx.x; b < kRadixBins; b += blockDim.x) old[b] = 0u;
                 }
-                sweep_radix_pick(sw->tk_hist[q % 3u], shift, width, sc.tk_prefix, sc.tk_remain);
+                sweep_radix_pick(A.sw->tk_hist[q % 3u], shift, width, sc.tk_prefix, sc.tk_remain);
                 if (threadIdx.x == 0) sc.tk_pass = q + 1u;
                 __syncthreads();
             }
@@ -1272,21 +1280,21 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
             if (mv.acc && mv.r > 2) {
                 NodeAcc<T> acc = kNoAcc<T>;
                 acc.pr = pow_share();
-                publish<T>(acc, &sw->slot[sc.p], ps, false);
+                publish<T>(acc, &A.sw->slot[sc.p], ps, false);
                 __syncthreads();  // (the scratch is used again; the selection clears cash)
             }
             if (threadIdx.x == 0) sm.next_group = 0;
-            if (threadIdx.x == 0) mv.n_pieces = &sw->slot[sc.p].pieces;
+            if (threadIdx.x == 0) mv.n_pieces = &A.sw->slot[sc.p].pieces;
             __syncthreads();
             NodeAcc<T> acc = kNoAcc<T>;
             if (sc.all) node_pass<T, kHasW, PASS_ALL>(A, mv, sc.ax, sm, acc);
             else node_pass<T, kHasW, PASS_SELECT>(A, mv, sc.ax, sm, acc);
-            publish<T>(acc, &sw->slot[sc.p], ps, mv.acc, &sm.n_list);
+            publish<T>(acc, &A.sw->slot[sc.p], ps, mv.acc, &sm.n_list);
         }
         {
             auto choose = [&]() {
                 // every total of the move in one round of loads
-                SweepSlot* sl = &sw->slot[sc.p];
+                SweepSlot* sl = &A.sw->slot[sc.p];
                 const double2 rts = ldcg_pair(&sl->reserve);
                 const double2 mm = ldcg_pair(&sl->msum);
                 const double2 apr = ldcg_pair(&sl->a);
@@ -1302,9 +1310,9 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
                 sc.n_pieces = (long long)np;
                 if (mv.acc) sc.now = (unsigned long long)__double_as_longlong(rts.y);
                 // every block is done with the last move's slot
-                if (blockIdx.x == 0) clear_slot(&sw->slot[rot3(rot3(sc.p))]);
+                if (blockIdx.x == 0) clear_slot(&A.sw->slot[rot3(rot3(sc.p))]);
             };
-            if (!grid_barrier_with(&sw->bar, sc.target, ctl.barrier_limit_ns,
+            if (!grid_barrier_with(&A.sw->bar, sc.target, ctl.barrier_limit_ns,
                                    blockIdx.x == 0 ? sc.ts[sc.tb] + 3 : nullptr, owed, choose))
                 goto aborted;
         }
@@ -1316,11 +1324,11 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
         } else if (sc.mode == MODE_PULL) {
             if (!sc.all && !mv.dense) {
                 dense_from_lists<T>(A, sm);
-                if (!grid_barrier(&sw->bar, sc.target, ctl.barrier_limit_ns)) goto aborted;
+                if (!grid_barrier(&A.sw->bar, sc.target, ctl.barrier_limit_ns)) goto aborted;
             }
             pull_tiles<T, T, kHasW, true, kSweepThreads>(A.c, A.mt, A.t_ptr, A.t_src, A.t_w, A.tile_r, A.tile_e,
                                                          A.ntiles, blockIdx.x, gridDim.x, sm.pull,
-                                                         &sw->slot[sc.p].chunk_next);
+                                                         &A.sw->slot[sc.p].chunk_next);
         }
         {
             // (the move's times stay until they are logged: the next move
@@ -1330,31 +1338,31 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
                 sc.tb ^= 1;
                 sc.ts[sc.tb][0] = sc.ts[sc.tb][1] = sc.ts[sc.tb][2] = sc.ts[sc.tb ^ 1][6];
             };
-            if (!grid_barrier_with(&sw->bar, sc.target, ctl.barrier_limit_ns,
+            if (!grid_barrier_with(&A.sw->bar, sc.target, ctl.barrier_limit_ns,
                                    blockIdx.x == 0 ? sc.ts[sc.tb] + 5 : nullptr, end_move, times))
                 goto aborted;
         }
         if (sc.leave) break;
     }
     if (lead) {
-        write_owed(sc, st, A.log);
-        st->l1 = sc.l1;
-        st->sumr = sc.sumr;
-        st->iters = sc.iters;
-        st->t_start = sc.t_start;
-        st->stall_mark = sc.stall_mark;
-        st->stall_count = sc.stall_count;
-        sw->bar.parity = (unsigned int)sc.p;
-        sw->bar.tk_pass = sc.tk_pass;
+        write_owed(sc, A.st, A.log);
+        A.st->l1 = sc.l1;
+        A.st->sumr = sc.sumr;
+        A.st->iters = sc.iters;
+        A.st->t_start = sc.t_start;
+        A.st->stall_mark = sc.stall_mark;
+        A.st->stall_count = sc.stall_count;
+        A.sw->bar.parity = (unsigned int)sc.p;
+        A.sw->bar.tk_pass = sc.tk_pass;
         if (sc.stop >= 0) {
-            st->done = 1;
-            st->status = sc.stop;
-            st->mode = MODE_NONE;
+            A.st->done = 1;
+            A.st->status = sc.stop;
+            A.st->mode = MODE_NONE;
         } else {
-            st->want_refresh = 1;
+            A.st->want_refresh = 1;
             if (sc.leave == 2) {  // the last test was of a cash to re-derive: no move
-                st->skip_move = 1;
-                st->mode = MODE_NONE;
+                A.st->skip_move = 1;
+                A.st->mode = MODE_NONE;
             }
         }
         if (A.use_cond) {
@@ -1366,8 +1374,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
 aborted:
     // A barrier wait gave up: end the solve with an error status.
     if (threadIdx.x == 0) {
-        st->done = 1;
-        st->status = ST_BARRIER;
+        A.st->done = 1;
+        A.st->status = ST_BARRIER;
         if (A.use_cond) {
             cudaGraphSetConditional(A.cond_loop, 0u);
             if (ctl.mixed) cudaGraphSetConditional(A.cond_refresh, 0u);
