@@ -470,11 +470,6 @@ static SweepArgs<T> sweep_args(rlgl_ctx* ctx, const Conds& cd) {
     a.deg = ctx->deg;
     a.list = (Green<T>*)ctx->f_list;
     a.pieces = (Piece<T>*)ctx->pieces;
-    // Links and what a move reads or writes once a node leave the L2 first
-    // where the nodes' cash, 1/d and history take most of it (129 MB):
-    // symmetrised R-MAT 24 (268 MB), a move 294 -> 234 us; R-MAT 20 (17 MB),
-    // 31.1 -> 32.8 us, so not there.
-    a.beyond_l2 = ctx->n * (long long)(2 * sizeof(T) + 8) > (96ll << 20) ? 1 : 0;
     a.n_hubs = ctx->n_hubs;
     a.hub1 = ctx->hub1;
     a.col = ctx->col;
@@ -500,14 +495,26 @@ static SweepArgs<T> sweep_args(rlgl_ctx* ctx, const Conds& cd) {
     return a;
 }
 
+// The sweep's kernel: where the nodes' cash, 1/d and history take most of the
+// L2 (129 MB), the one in which links and what a move reads or writes once a
+// node leave the L2 first. Symmetrised R-MAT 24 (268 MB), a move 294 -> 234
+// us. Elsewhere what it reads stays in L1 and L2 for the next move. With one
+// kernel for both, the policy an operand: R-MAT 20 (17 MB) 2772 against 2708
+// us, 281903 nodes FP64 7425 against 7054, PageRank of 500000 nodes 3300
+// against 3238.
+template <typename T>
+static void (*sweep_kernel(const rlgl_ctx* ctx))(SweepArgs<T>) {
+    const bool far = ctx->n * (long long)(2 * sizeof(T) + 8) > (96ll << 20);
+    if (far) return ctx->has_w ? k_far_sweep<T, true> : k_far_sweep<T, false>;
+    return ctx->has_w ? k_sweep<T, true> : k_sweep<T, false>;
+}
+
 template <typename T>
 static rlgl_status enqueue_sweep(Launch L, const Conds& cd) {
     rlgl_ctx* ctx = L.ctx;
     const SweepArgs<T> a = sweep_args<T>(ctx, cd);
-    if (ctx->has_w)
-        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_sweep, kSweepThreads, sizeof(SweepSmem<T>), k_sweep<T, true>, a))));
-    else
-        LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_sweep, kSweepThreads, sizeof(SweepSmem<T>), k_sweep<T, false>, a))));
+    LAUNCH(L, KC_SWEEP, TRY((launch_coop<T>(ctx, ctx->grid_sweep, kSweepThreads, sizeof(SweepSmem<T>),
+                                            sweep_kernel<T>(ctx), a))));
     return RLGL_OK;
 }
 
@@ -614,21 +621,17 @@ static int bsweep_fit(rlgl_ctx* ctx, int bt) {
 // Blocks of the sweep: all that fit on the device at once (the occupancy of
 // the instantiation this context uses), fewer for a small chain, where each
 // block still gets at least one block-iteration of nodes.
-template <typename T, bool kHasW>
-static int sweep_fit_t() {
+template <typename T>
+static int sweep_fit(rlgl_ctx* ctx) {
     int nb = 0;
     constexpr int smem = (int)sizeof(SweepSmem<T>);
-    if (cudaFuncSetAttribute(k_sweep<T, kHasW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_sweep<T, kHasW>, kSweepThreads, smem) != cudaSuccess) {
+    void (*const kernel)(SweepArgs<T>) = sweep_kernel<T>(ctx);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kSweepThreads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return nb;
-}
-
-template <typename T>
-static int sweep_fit(rlgl_ctx* ctx) {
-    return ctx->has_w ? sweep_fit_t<T, true>() : sweep_fit_t<T, false>();
 }
 
 static int sweep_grid(rlgl_ctx* ctx) {

@@ -268,12 +268,10 @@ __device__ __forceinline__ void red_add(double* p, double v) {
 
 // Loads of links, which a pass over them reads once: first to leave the L2
 // (and not kept in L1), so that the node values gathered or added to stay.
-// (first: whether they are first to leave; else as any load)
-__device__ __forceinline__ unsigned long long stream_policy(bool first = true) {
-    unsigned long long p, q;
+__device__ __forceinline__ unsigned long long stream_policy() {
+    unsigned long long p;
     asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(q));
-    return first ? p : q;
+    return p;
 }
 __device__ __forceinline__ int ld_stream(const int* p, unsigned long long pol) {
     int v;
@@ -291,18 +289,24 @@ __device__ __forceinline__ double ld_stream(const double* p, unsigned long long 
     return v;
 }
 // The same for links read in short runs, whose sectors neighbouring rows
-// share: kept in L1.
+// share: kept in L1 (kFirst: first to leave the L2; else as any load).
+template <bool kFirst>
 __device__ __forceinline__ int ld_run(const int* p, unsigned long long pol) {
+    if (!kFirst) return __ldg(p);
     int v;
     asm("ld.global.nc.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
     return v;
 }
+template <bool kFirst>
 __device__ __forceinline__ float ld_run(const float* p, unsigned long long pol) {
+    if (!kFirst) return __ldg(p);
     float v;
     asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
     return v;
 }
-__device__ __forceinline__ void red_add_stream(double* p, double v, unsigned long long pol) {
+template <bool kFirst>
+__device__ __forceinline__ void red_add(double* p, double v, unsigned long long pol) {
+    if (!kFirst) return red_add(p, v);
     asm volatile("red.global.add.L2::cache_hint.f64 [%0], %1, %2;" ::"l"(p), "d"(v), "l"(pol) : "memory");
 }
 

@@ -217,7 +217,6 @@ struct SweepArgs {
     const int* deg;     // links of each row
     Green<T>* list;     // the sweep's green rows, each block's in its own part
     Piece<T>* pieces;   // pieces of its long green rows
-    int beyond_l2;  // the node arrays do not fit the L2 (see sweep_args)
     int n_hubs;  // hub targets of the push, and the only one when there is one
     int hub1;
     const int* rank;  // source order of mt and mt2 (see source_of)
@@ -420,19 +419,19 @@ __device__ __forceinline__ void add_edges(T* __restrict__ c, int (&j)[kU], const
 
 // Pushes the links [pos, pos + len) of one row by the whole warp, four
 // links a lane in flight.
-template <typename T, bool kHasW>
+template <typename T, bool kHasW, bool kFar>
 __device__ __forceinline__ void push_row(const SweepArgs<T>& A, long long pos, int len, T m, HotSmem<T>& hot) {
     const int lane = threadIdx.x & 31;
-    const unsigned long long pol = stream_policy(A.beyond_l2);
+    const unsigned long long pol = stream_policy();
     for (int o = 0; o < len; o += 128) {
         int j[4];
         T v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int e = o + q * 32 + lane;
-            j[q] = e < len ? ld_run(A.col + pos + e, pol) : -1;
+            j[q] = e < len ? ld_run<kFar>(A.col + pos + e, pol) : -1;
             v[q] = m;
-            if (kHasW && e < len) v[q] = m * (T)ld_run(A.w + pos + e, pol);
+            if (kHasW && e < len) v[q] = m * (T)ld_run<kFar>(A.w + pos + e, pol);
         }
         add_edges<T, 4>(A.c, j, v, A.n_hubs, A.hub1, hot);
     }
@@ -499,7 +498,7 @@ enum Pass : int { PASS_STATS, PASS_SELECT, PASS_ALL };
 // counter in shared memory (zero at the start of a pass; warp w starts with
 // group w): weighted R-MAT 22, 12 moves, 2788 -> 2766 us. The next group's
 // cash is loaded before the current one is listed.
-template <typename T, bool kHasW, int kPass>
+template <typename T, bool kHasW, bool kFar, int kPass>
 __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<T>& mv, const SchedAux& ax,
                                           SweepSmem<T>& sm, NodeAcc<T>& acc) {
     constexpr int kV = NodeVec<T>::kV;
@@ -518,7 +517,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
             C[q] = idg[q] = T(0);
             if (q * 32 < group && i < n) {
                 C[q] = __ldcg(A.c + i);
-                if (need_idg) idg[q] = ld_stream(reinterpret_cast<const T*>(A.ideg) + i, stream_policy(A.beyond_l2));
+                if (need_idg) idg[q] = kFar ? ld_stream(A.ideg + i, stream_policy()) : __ldg(A.ideg + i);
             }
         }
     };
@@ -578,7 +577,8 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
             deg[q] = 0;
             if (gm >> q & 1u) {
                 m[q] = C[q] * (scale_is_idg ? idg[q] : __ldg(scale + i));
-                if (kPass == PASS_SELECT) deg[q] = need_idg ? degree_of(idg[q], A.deg + i) : __ldg(A.deg + i);
+                // (unit weights: see push_rows)
+                if (kPass == PASS_SELECT) deg[q] = (kFar ? need_idg : scale_is_idg) ? degree_of(idg[q], A.deg + i) : __ldg(A.deg + i);
             }
         }
 #pragma unroll
@@ -588,7 +588,7 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
             acc.m += C[q];
             acc.ma += fabs(C[q]);
             A.c[i] = T(0);
-            red_add_stream(A.H + i, widen(C[q]), stream_policy(A.beyond_l2));  // no load: the L2 adds
+            red_add<kFar>(A.H + i, widen(C[q]), stream_policy());  // no load: the L2 adds
         }
         if (kPass == PASS_ALL || mv.dense) {
 #pragma unroll
@@ -662,7 +662,7 @@ __device__ __noinline__ T pow_sum(const T* c, const T* ideg, int n, int r) {
 // as the number of rows that begin at or before it (one warp-wide or and a
 // bit count). Four windows are in flight. The block's rows of more than
 // kShortRow links come last, one warp each.
-template <typename T, bool kHasW>
+template <typename T, bool kHasW, bool kFar>
 __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& sm, int np) {
     const int lane = threadIdx.x & 31;
     const unsigned int upto = 0xffffffffu >> (31 - lane);
@@ -671,9 +671,9 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
         const long long pos = __ldcg(&A.pieces[p].pos);
         const int len = __ldcg(&A.pieces[p].len);
         const T m = __ldcg(&A.pieces[p].m);
-        push_row<T, kHasW>(A, pos, len, m, sm.hot);
+        push_row<T, kHasW, kFar>(A, pos, len, m, sm.hot);
     }
-    const unsigned long long pol = stream_policy(A.beyond_l2);
+    const unsigned long long pol = stream_policy();
     const int nl = sm.n_list;
     const OwnNodes<T> own(A.n);
     for (;;) {
@@ -689,7 +689,9 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
             const int id = __ldcg(&e->id);
             m = __ldcg(&e->m);
             base = __ldg(A.row_ptr + id);
-            len = (int)(__ldg(A.row_ptr + id + 1) - base);
+            // (from both offsets where the selection took the degree from
+            // 1/d; else the degree is in L1 since)
+            len = kFar || (sizeof(T) == 4 && !kHasW) ? (int)(__ldg(A.row_ptr + id + 1) - base) : __ldg(A.deg + id);
             if (len > kHubRow) len = 0;  // in pieces
         }
         const unsigned int mid = __ballot_sync(0xffffffffu, len > kShortRow);
@@ -740,8 +742,8 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
                 const long long pos = __shfl_sync(0xffffffffu, base, k) + e;
                 v[q] = __shfl_sync(0xffffffffu, m, k);
                 if (e < E) {
-                    j[q] = ld_run(A.col + pos, pol);
-                    if (kHasW) v[q] *= (T)ld_run(A.w + pos, pol);
+                    j[q] = ld_run<kFar>(A.col + pos, pol);
+                    if (kHasW) v[q] *= (T)ld_run<kFar>(A.w + pos, pol);
                 }
             }
             add_edges<T, 4>(A.c, j, v, A.n_hubs, A.hub1, sm.hot);
@@ -754,7 +756,7 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
         if (lane == 0) z = atomicAdd(&sm.next_mid, 1);
         z = __shfl_sync(0xffffffffu, z, 0);
         if (z >= nm) break;
-        push_row<T, kHasW>(A, sm.mid.base[z], sm.mid.len[z], sm.mid.m[z], sm.hot);
+        push_row<T, kHasW, kFar>(A, sm.mid.base[z], sm.mid.len[z], sm.mid.m[z], sm.hot);
     }
 }
 
@@ -1024,8 +1026,8 @@ __device__ __forceinline__ void publish(const NodeAcc<T>& acc, SweepSlot* sl, Pu
     }
 }
 
-template <typename T, bool kHasW>
-__global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
+template <typename T, bool kHasW, bool kFar>
+__device__ __forceinline__ void sweep_moves(const SweepArgs<T>& A) {
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
     if (A.st->done) {
         if (A.use_cond && lead) cudaGraphSetConditional(A.cond_loop, 0u);
@@ -1185,7 +1187,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
             // ------------------------------------------ stats and control
             {
                 NodeAcc<T> acc = kNoAcc<T>;
-                node_pass<T, kHasW, PASS_STATS>(A, mv, sc.ax, sm, acc);
+                node_pass<T, kHasW, kFar, PASS_STATS>(A, mv, sc.ax, sm, acc);
                 if (mv.r > 2) acc.pr = pow_share();
                 publish<T>(acc, &A.sw->slot[sc.p], ps, true);
             }
@@ -1287,8 +1289,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
             if (threadIdx.x == 0) mv.n_pieces = &A.sw->slot[sc.p].pieces;
             __syncthreads();
             NodeAcc<T> acc = kNoAcc<T>;
-            if (sc.all) node_pass<T, kHasW, PASS_ALL>(A, mv, sc.ax, sm, acc);
-            else node_pass<T, kHasW, PASS_SELECT>(A, mv, sc.ax, sm, acc);
+            if (sc.all) node_pass<T, kHasW, kFar, PASS_ALL>(A, mv, sc.ax, sm, acc);
+            else node_pass<T, kHasW, kFar, PASS_SELECT>(A, mv, sc.ax, sm, acc);
             publish<T>(acc, &A.sw->slot[sc.p], ps, mv.acc, &sm.n_list);
         }
         {
@@ -1319,7 +1321,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
 
         // ----------------------------------------------------------- move
         if (sc.mode == MODE_PUSH) {
-            push_rows<T, kHasW>(A, sm, (int)sc.n_pieces);
+            push_rows<T, kHasW, kFar>(A, sm, (int)sc.n_pieces);
             if (A.n_hubs) flush_hubs<T>(A, sm.hot);
         } else if (sc.mode == MODE_PULL) {
             if (!sc.all && !mv.dense) {
@@ -1381,6 +1383,17 @@ aborted:
             if (ctl.mixed) cudaGraphSetConditional(A.cond_refresh, 0u);
         }
     }
+}
+
+template <typename T, bool kHasW>
+__global__ void __launch_bounds__(kSweepThreads, 1) k_sweep(SweepArgs<T> A) {
+    sweep_moves<T, kHasW, false>(A);
+}
+
+// Chains whose node arrays take most of the L2 (see sweep_kernel).
+template <typename T, bool kHasW>
+__global__ void __launch_bounds__(kSweepThreads, 1) k_far_sweep(SweepArgs<T> A) {
+    sweep_moves<T, kHasW, true>(A);
 }
 
 }  // namespace rlgl
