@@ -644,8 +644,18 @@ static int sweep_grid(rlgl_ctx* ctx) {
     return (int)(want < fit ? want : fit);
 }
 
-// Blocks of the power sweep: all that fit, fewer when the chain has fewer
-// merge-path tiles (and node block-iterations) than that.
+// Blocks of the power sweep (one an SM). A small chain's do not take the
+// whole GPU, where its solve may be one of several at once: four tiles a
+// warp, or two where that takes no more than a sixth of the SMs, and at most
+// half of the SMs until four tiles a warp would take two thirds of them.
+// Measured, us a solve of 100 moves alone / one of twelve at once, MIXED, for
+// one block in 3072 nodes; a block in 2048 rows and links; this rule:
+//    20000 nodes  3353 / 309;  1422 / 1241;  1928 / 280
+//    60000        3452 / 531;     - / -   ;  2703 / 678
+//   100000        3571 / 938;  2026 / -   ;  2841 / 1361
+//   200000        3581 / 1845; 2478 / -   ;  2501 / 2389
+// and FP64  20000 4625 / 409;  1405 / 1297;  2316 / 386
+//          200000 5069 / 2577; 3059 / -   ;  3053 / 2974
 template <typename T, bool kHasW>
 static int power_fit_t() {
     int nb = 0;
@@ -667,10 +677,11 @@ static int power_grid(rlgl_ctx* ctx) {
     const int nb = ctx->prec == RLGL_MIXED ? power_fit<float>(ctx) : power_fit<double>(ctx);
     if (nb < 1) return 0;
     const long long fit = (long long)nb * ctx->sms;
-    long long want = ctx->ntiles;
-    const long long nodes = (ctx->n + 4 * kPowThreads - 1) / (4 * kPowThreads);
-    if (nodes > want) want = nodes;
-    if (want < 1) want = 1;
+    const long long two = (ctx->nwtiles + 2 * kPowWarps - 1) / (2 * kPowWarps);
+    long long want = (two + 1) / 2;
+    if (want < ctx->sms / 6) want = two < ctx->sms / 6 ? two : ctx->sms / 6;
+    if (3 * want > 2 * ctx->sms) return (int)fit;
+    if (2 * want > ctx->sms) want = ctx->sms / 2;
     return (int)(want < fit ? want : fit);
 }
 
@@ -917,7 +928,6 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
     ctx->grid_push = grid_for(nnz, kPushChunk, ctx->sms * 4);
     ctx->grid_pull = grid_for(n + nnz, kMpItems, ctx->sms * 8);
     ctx->grid_sweep = sweep_grid(ctx);
-    ctx->grid_power = power_grid(ctx);
     const size_t cs = cash_size(ctx);
 
     TRY(dalloc(ctx, &ctx->row_ptr, (size_t)n + 1));
@@ -934,6 +944,7 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
     TRY(dalloc(ctx, &ctx->tile_e, (size_t)ctx->ntiles + 1));
     const long long witems = 32 * power_ipt((int)cs);
     ctx->nwtiles = (n + nnz + witems - 1) / witems;
+    ctx->grid_power = power_grid(ctx);  // (from the tile count)
     TRY(dalloc(ctx, &ctx->wtile_r, (size_t)ctx->nwtiles + 1));
     TRY(dalloc(ctx, &ctx->wtile_e, (size_t)ctx->nwtiles + 1));
     TRY(dalloc_bytes(ctx, &ctx->c, (size_t)n * cs));
