@@ -312,8 +312,11 @@ template <typename T>
 struct HotSmem {
     int hub[kHubSlots];
     double hot[kHubSlots];  // zero at rest
-    // with a single hub: the threads' sums (see hub_add), zero at rest
-    typename std::conditional<std::is_same<T, float>::value, float2, double>::type one[kSweepThreads];
+    // with a single hub: the threads' sums, zero at rest. (In shared memory:
+    // few chains have a hub, and the node loops need their registers. As a
+    // pair of FP32 numbers with the roundings carried along, PageRank of
+    // 500000 nodes takes as long: 3301 and 3300 us.)
+    double one[kSweepThreads];
 };
 
 // Rows of kShortRow < links <= kHubRow met by the block's push, left for
@@ -364,20 +367,6 @@ struct NodeAcc {
 template <typename T>
 constexpr NodeAcc<T> kNoAcc = {T(0), T(0), T(0), T(0), 0ull};
 
-// Adds v to a single hub target's sum of one thread: FP32 terms as a pair
-// of FP32 numbers whose sum carries every rounding error of the additions
-// (Knuth's two-sum), so that the FP64 pipe is left out of the edge loop;
-// FP64 terms in FP64. In shared memory: few chains have a hub, and the node
-// loops need their registers.
-__device__ __forceinline__ void hub_add(float2& h, float v) {
-    const float s = h.x, t = __fadd_rn(s, v), z = __fsub_rn(t, s);
-    h.y = __fadd_rn(h.y, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z)));
-    h.x = t;
-}
-__device__ __forceinline__ void hub_add(double& h, double v) { h += v; }
-__device__ __forceinline__ double hub_value(const float2& h) { return (double)h.x + (double)h.y; }
-__device__ __forceinline__ double hub_value(const double& h) { return h; }
-
 // The additions of kU edges a lane (target j, -1: none; amount v) to the
 // cash. Targets in the hub table (PageRank's auxiliary node, which
 // every node feeds) are summed apart: one of them by thread, several by warp
@@ -392,7 +381,7 @@ __device__ __forceinline__ void add_edges(T* __restrict__ c, int (&j)[kU], const
     } else if (n_hubs == 1) {
 #pragma unroll
         for (int q = 0; q < kU; ++q) {
-            if (j[q] == hub1) hub_add(hot.one[threadIdx.x], v[q]);
+            if (j[q] == hub1) hot.one[threadIdx.x] += (double)v[q];
             else if (j[q] >= 0) red_add(c + j[q], v[q]);
         }
     } else {
@@ -441,9 +430,9 @@ __device__ __forceinline__ void push_row(const SweepArgs<T>& A, long long pos, i
 template <typename T>
 __device__ __forceinline__ void flush_hubs(const SweepArgs<T>& A, HotSmem<T>& hot) {
     if (A.n_hubs == 1) {
-        const double x = warp_sum(hub_value(hot.one[threadIdx.x]));
+        const double x = warp_sum(hot.one[threadIdx.x]);
         if ((threadIdx.x & 31) == 0 && x != 0.0) atomicAdd(&hot.hot[hub_slot(A.hub1)], x);
-        hot.one[threadIdx.x] = {};
+        hot.one[threadIdx.x] = 0.0;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < kHubSlots; t += blockDim.x)
@@ -1051,7 +1040,7 @@ __device__ __forceinline__ void sweep_moves(const SweepArgs<T>& A) {
             sm.hot.hub[k] = A.n_hubs ? __ldg(A.hubs + k) : -1;
             sm.hot.hot[k] = 0.0;
         }
-        sm.hot.one[threadIdx.x] = {};
+        sm.hot.one[threadIdx.x] = 0.0;
     }
     __syncthreads();
     const int n = A.n;
