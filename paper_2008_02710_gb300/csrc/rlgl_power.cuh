@@ -83,16 +83,24 @@ __host__ __device__ constexpr int power_ipt(int cash_bytes) { return cash_bytes 
 
 // Shared memory of one warp of the power sweep: its merge-path tile (the
 // gathered in-link values, the row ends) and each row's in-link sum (local
-// row index). With FP32 cash the sums take the place of the ends: a row's
-// end is last read before the sum is there (see power_tiles).
+// row index). With FP32 cash the bits of a sum take the place of the row's
+// end: that is last read before the sum is there (see power_tiles).
 template <typename T>
 struct PowWarp {
     static constexpr int kItems = 32 * power_ipt((int)sizeof(T));
-    static constexpr bool kShare = sizeof(T) == sizeof(int);
     T val[kItems];
     int ends[kItems + 1];
-    T sums[kShare ? 1 : kItems];
-    __device__ __forceinline__ T* rsum() { return kShare ? reinterpret_cast<T*>(ends) : sums; }
+    T sums[kItems];
+    __device__ __forceinline__ T sum(int k) const { return sums[k]; }
+    __device__ __forceinline__ void set_sum(int k, T v) { sums[k] = v; }
+};
+template <>
+struct PowWarp<float> {
+    static constexpr int kItems = 32 * power_ipt((int)sizeof(float));
+    float val[kItems];
+    int ends[kItems + 1];
+    __device__ __forceinline__ float sum(int k) const { return __int_as_float(ends[k]); }
+    __device__ __forceinline__ void set_sum(int k, float v) { ends[k] = __float_as_int(v); }
 };
 
 // Hot sources kept in shared memory, and the block's dynamic shared memory.
@@ -217,7 +225,6 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
     constexpr int kPowIpt = power_ipt((int)sizeof(T));
     const int lane = threadIdx.x & 31;
     PowWarp<T>& ws = sm.warp[threadIdx.x >> 5];
-    T* const rsum = ws.rsum();
     const unsigned long long pol = stream_policy();
     // (tiles: at most 2^38 / 256, an int; rows: below 2^27)
     const int ntiles = (int)A.nwtiles;
@@ -311,9 +318,10 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
             j = d - lo;
             row_start = (i == 0) ? start0 : ws.ends[i - 1];
         }
-        // From here on a lane uses only the ends of rows of which it holds an
+        // From here on a lane reads only the ends of rows of which it holds an
         // item, and writes in this loop only sums of rows that lie in it
-        // whole: no other lane holds an item of those.
+        // whole: no other lane holds an item of those. Every other sum is
+        // written once all lanes have left the loop.
         __syncwarp();
         if (d < total) {
             bool whole = (j == row_start);  // no in-link of row i before this lane
@@ -324,7 +332,7 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
                 if (d + q < total) {
                     const bool link = j < end;
                     if (link) sum += ws.val[j];
-                    if (!link && whole) rsum[i] = sum;  // a row with no in-link sums to zero
+                    if (!link && whole) ws.set_sum(i, sum);  // a row with no in-link sums to zero
                     if (!link && !whole) {
                         rowA = i;
                         accA = sum;
@@ -333,7 +341,8 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
                         sum = T(0);
                         j0 = j;
                         ++i;
-                        end = ws.ends[i];
+                        // (the next item's row, or past the last of the tile, which none writes)
+                        if (q + 1 < kPowIpt) end = ws.ends[i];
                         whole = true;
                     }
                     j += link ? 1 : 0;
@@ -344,6 +353,7 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
                 accB = sum;
             }
         }
+        __syncwarp();
         const T run = warp_segscan<T>(rowB, accB);
         const int pkey = __shfl_up_sync(0xffffffffu, rowB, 1);
         const T pval = __shfl_up_sync(0xffffffffu, run, 1);
@@ -354,7 +364,7 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
             if (rowA == 0 && first_split)
                 atomicAdd(A.facc + t.r0, sum);  // finished after the barrier
             else
-                rsum[rowA] = sum;
+                ws.set_sum(rowA, sum);
         }
         const int last = (total - 1) / kPowIpt;
         if (lane == last && rowB >= 0) atomicAdd(A.facc + t.r0 + rowB, run);
@@ -365,9 +375,9 @@ __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __re
         for (int k = lane; k < t.nr; k += 32) {
             if (k == 0 && first_split) continue;
             if (k == lane)
-                power_row_with<T>(A, mt_next, t.r0 + k, rsum[k], oldv, scv, acc);
+                power_row_with<T>(A, mt_next, t.r0 + k, ws.sum(k), oldv, scv, acc);
             else
-                power_row<T>(A, mt_next, t.r0 + k, rsum[k], acc);
+                power_row<T>(A, mt_next, t.r0 + k, ws.sum(k), acc);
         }
         __syncwarp();  // the warp's shared memory is rewritten next
         b = bn;
