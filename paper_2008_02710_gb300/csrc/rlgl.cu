@@ -124,9 +124,9 @@ struct rlgl_ctx {
     int* hubs = nullptr;  // hub table of the push (kHubSlots ids, -1 empty), null when none
     int n_hubs = 0;
     int hub1 = -1;        // the hub when there is one
-    int* deg = nullptr;      // links of each row
-    int* rank = nullptr;     // source order of the in-link copy (see source_of); null for a batch
-    HotInfo* hot = nullptr;  // its hot front
+    int* deg = nullptr;    // links of each row, then (single chains) rank and n_hot
+    int* rank = nullptr;   // source order of the in-link copy (see source_of); null for a batch
+    int* n_hot = nullptr;  // length of its hot front
     void* f_list = nullptr;  // the phase kernels' f_eoff and f_base; the sweep's list of green rows
     void* pieces = nullptr;  // pieces of the long green rows of a move (sweep)
     // profiling
@@ -462,7 +462,7 @@ static SweepArgs<T> sweep_args(rlgl_ctx* ctx, const Conds& cd) {
     a.ideg = (const T*)ctx->ideg;
     a.masks = ctx->masks;
     a.rank = ctx->rank;
-    a.hot = ctx->hot;
+    a.n_hot = ctx->n_hot;
     a.mt = (T*)ctx->mt;
     a.mt2 = (T*)ctx->hsrc;  // free while no re-derivation runs
     a.facc = (T*)ctx->f_m;  // the power sweep clears it at every launch
@@ -490,7 +490,6 @@ static SweepArgs<T> sweep_args(rlgl_ctx* ctx, const Conds& cd) {
     a.cond_refresh = cd.refresh;
     a.use_cond = cd.use;
     a.n = (int)ctx->n;
-    a.vec_ok = vec_aligned(ctx);
     a.hubs = ctx->n_hubs ? ctx->hubs : nullptr;
     return a;
 }
@@ -953,21 +952,25 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
     TRY(dalloc(ctx, &ctx->y, (size_t)n));
     TRY(dalloc(ctx, &ctx->hsrc, (size_t)n));
     TRY(dalloc(ctx, &ctx->colsum, (size_t)n));
-    TRY(dalloc_bytes(ctx, &ctx->f_list, 2 * (size_t)n * sizeof(long long)));
+    TRY(dalloc_bytes(ctx, &ctx->f_list, 2 * (size_t)n * sizeof(long long) + pieces_bytes(nnz, cs)));
     ctx->f_eoff = (long long*)ctx->f_list;
     ctx->f_base = ctx->f_eoff + n;
-    TRY(dalloc(ctx, &ctx->deg, (size_t)n));
+    ctx->pieces = ctx->f_base + n;
+    TRY(dalloc(ctx, &ctx->deg, batch ? (size_t)n : 2 * (size_t)n + 1));
+    if (!batch) {
+        ctx->rank = ctx->deg + n;
+        ctx->n_hot = ctx->rank + n;
+    }
     TRY(dalloc_bytes(ctx, &ctx->f_m, (size_t)n * cs));
     TRY(dalloc(ctx, &ctx->chunk_row, (size_t)(nnz / kPushChunk + 2)));
     TRY(dalloc(ctx, &ctx->part, (size_t)(4 * kMaxGrid + 8)));
-    TRY(dalloc_bytes(ctx, &ctx->pieces, pieces_bytes(nnz, cs)));
     TRY(dalloc(ctx, &ctx->err, 1));
     TRY(dalloc(ctx, &ctx->log, (size_t)kLogCap));
     TRY(dalloc(ctx, &ctx->st, 1));
     TRY(dalloc(ctx, &ctx->sw, 1));
     // the sweep reads slot fields in 16-byte pairs (pool allocations are
     // aligned far beyond that)
-    if ((((uintptr_t)ctx->sw | (uintptr_t)ctx->pieces | (uintptr_t)ctx->f_list) & 15u) != 0)
+    if ((((uintptr_t)ctx->sw | (uintptr_t)ctx->f_list) & 15u) != 0)
         return fail(ctx, RLGL_ENOMEM, "device buffers not 16-byte aligned");
     ctx->host_st = static_cast<DevState*>(pin_get());
     if (!ctx->host_st) return fail(ctx, RLGL_ENOMEM, "pinned host allocation failed");
@@ -982,7 +985,12 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
     if (ctx->has_w) TRY(upload(ctx, ctx->w, w, (size_t)nnz * sizeof(float), src));
 
     const int gv = grid_for(nnz, kThreads, ctx->sms * 16);
-    k_validate<<<gv, kThreads, 0, ctx->stream>>>(ctx->row_ptr, ctx->col, ctx->w, n, nnz, ctx->err);
+    // (the log, which the first move writes, is scratch until then)
+    static_assert(HotScratch::bytes(hot_cap(4)) <= (size_t)kLogCap * sizeof(MoveRecord), "the log holds the scratch");
+    const int cap_hot = hot_cap((int)cs);
+    const HotScratch hs(ctx->log, cap_hot);
+    k_validate<<<gv, kThreads, 0, ctx->stream>>>(ctx->row_ptr, ctx->col, ctx->w, n, nnz, ctx->err, hs.hist,
+                                                 batch ? 0 : HotScratch::kZero);
     CKL(ctx);
     unsigned int err = 0;
     CK(ctx, cudaMemcpyAsync(&err, ctx->err, sizeof err, cudaMemcpyDeviceToHost, ctx->stream));
@@ -1008,22 +1016,14 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
         CKL(ctx);
     }
     // Source order of the in-link copy (a batch's pulls stay in node order):
-    // the hot sources for the all-green sweep's shared memory.
+    // the hot sources for the all-green sweep's shared memory. hsrc: s in it.
     if (!batch) {
-        TRY(dalloc(ctx, &ctx->rank, (size_t)n));
-        TRY(dalloc(ctx, &ctx->hot, 1));
-        unsigned int* hist = nullptr;
-        TRY(dalloc(ctx, &hist, (size_t)kHotBins + 2 * (size_t)hot_cap(4)));
-        int* la = (int*)hist + kHotBins;
-        int* lb = la + hot_cap(4);
-        CK(ctx, cudaMemsetAsync(ctx->hot, 0, sizeof(HotInfo), ctx->stream));
-        CK(ctx, cudaMemsetAsync(hist, 0, kHotBins * sizeof(unsigned int), ctx->stream));
-        const int gh = grid_for(n, 1024, ctx->sms);
-        k_degree_hist<<<gh, 1024, 0, ctx->stream>>>(ctx->deg, (int)n, hist);
-        k_hot_lists<<<gh, 1024, 0, ctx->stream>>>(ctx->deg, (int)n, hist, hot_cap((int)cs), ctx->hot, ctx->rank, la, lb);
-        k_hot_swap<<<grid_for(hot_cap((int)cs), kThreads, ctx->sms), kThreads, 0, ctx->stream>>>(ctx->hot, la, lb, ctx->rank);
+        k_degree_hist<<<grid_for(n, 1024, ctx->sms), 1024, 0, ctx->stream>>>(ctx->deg, (int)n, hs.hist);
+        k_hot_lists<<<grid_for(n, 1024, 2 * ctx->sms), 1024, 0, ctx->stream>>>(
+            ctx->deg, (int)n, hs, cap_hot, ctx->n_hot, ctx->rank, ctx->s, ctx->hsrc);
+        k_hot_swap<<<grid_for(cap_hot < n ? cap_hot : n, kThreads, ctx->sms), kThreads, 0, ctx->stream>>>(
+            hs, ctx->rank, ctx->hsrc);
         CKL(ctx);
-        dfree(ctx, hist);
     }
     // In-link (CSC) copy: counts, scan, scatter.
     long long* cursor = nullptr;
@@ -1132,13 +1132,13 @@ static rlgl_status create_common(int64_t n, int64_t nnz, const int64_t* row_ptr,
                                                       ctx->wtile_e);
     CKL(ctx);
     CK(ctx, cudaMemsetAsync(ctx->colsum, 0, (size_t)n * sizeof(double), ctx->stream));
-    k_to_source_order<<<ctx->grid_nodes, kThreads, 0, ctx->stream>>>(ctx->s, ctx->rank, (int)n, ctx->hsrc);
+    const double* s_src = batch ? ctx->s : ctx->hsrc;
     if (ctx->has_w)
         k_colsum_tiles<true><<<ctx->grid_pull, kThreads, 0, ctx->stream>>>(
-            ctx->colsum, ctx->hsrc, ctx->t_ptr, ctx->t_src, ctx->t_w, ctx->tile_r, ctx->tile_e, ctx->ntiles);
+            ctx->colsum, s_src, ctx->t_ptr, ctx->t_src, ctx->t_w, ctx->tile_r, ctx->tile_e, ctx->ntiles);
     else
         k_colsum_tiles<false><<<ctx->grid_pull, kThreads, 0, ctx->stream>>>(
-            ctx->colsum, ctx->hsrc, ctx->t_ptr, ctx->t_src, ctx->t_w, ctx->tile_r, ctx->tile_e, ctx->ntiles);
+            ctx->colsum, s_src, ctx->t_ptr, ctx->t_src, ctx->t_w, ctx->tile_r, ctx->tile_e, ctx->ntiles);
     CKL(ctx);
     if (eager_graph && ctx->params.persistent && build_sweep_graph(ctx, false) != RLGL_OK) {
         // (the first solve tries again and falls back to the phase kernels)
@@ -2060,7 +2060,7 @@ int64_t rlgl_footprint(int64_t n, int64_t nnz, int32_t weighted, rlgl_precision 
     int64_t b = 0;
     b += 2 * ((n + 1) * 8 + nnz * 4 + (weighted ? nnz * 4 : 0));  // CSR and CSC
     b += n * (8 + (prec == RLGL_MIXED ? 4 : 0) + cs + 4);            // s, sf, 1/deg, deg
-    if (n_chains <= 1) b += n * 4 + (int64_t)sizeof(HotInfo);        // source order
+    if (n_chains <= 1) b += (n + 1) * 4;                              // source order
     b += 2 * (ntiles + 1) * 8 + 2 * (nwtiles + 1) * 8;               // merge-path tiles (block, warp)
     b += n * (cs + 8 + cs + 8 + 8 + 8 + 8 + cs + 8);                 // c H mt y hsrc f_eoff f_base f_m colsum
     b += (nnz / kPushChunk + 2) * 4;                                 // chunk index
@@ -2104,10 +2104,9 @@ void rlgl_destroy(rlgl_ctx* ctx) {
     void* dev[] = {ctx->row_ptr, ctx->col, ctx->w, ctx->s, ctx->sf, ctx->ideg, ctx->t_ptr, ctx->t_src, ctx->t_w,
                    ctx->tile_r, ctx->tile_e, ctx->wtile_r, ctx->wtile_e, ctx->c, ctx->H, ctx->mt, ctx->y, ctx->hsrc, ctx->c0,
                    ctx->colsum,
-                   ctx->f_list, ctx->deg, ctx->rank, ctx->hot, ctx->f_m, ctx->chunk_row, ctx->part, ctx->masks,
+                   ctx->f_list, ctx->deg, ctx->f_m, ctx->chunk_row, ctx->part, ctx->masks,
                    ctx->err, ctx->log, ctx->st, ctx->sw, ctx->node_ptr, ctx->chain_of, ctx->cs,
-                   ctx->bsums, ctx->ct_off, ctx->ct_r, ctx->ct_e, ctx->grp, ctx->bq, ctx->q_next, ctx->hubs,
-                   ctx->pieces};
+                   ctx->bsums, ctx->ct_off, ctx->ct_r, ctx->ct_e, ctx->grp, ctx->bq, ctx->q_next, ctx->hubs};
     for (void* p : dev)
         dfree(ctx, p);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);

@@ -900,13 +900,25 @@ __device__ __forceinline__ int source_of(const int* __restrict__ rank, int i) { 
 
 constexpr int kHotBins = 4096;      // out-degrees counted one by one below this
 constexpr int kHotMinDegree = 64;   // a hot source saves that many gathers a pull over the GPU and costs one load per SM
-struct HotInfo {
-    int thr;    // hot: out-degree >= thr
-    int count;  // hot sources
-    int na, nb; // nodes displaced, and hot nodes to move to the front
+// Scratch of the source order: the histogram of the out-degrees (those of
+// kHotBins - 1 and more together; zero before k_degree_hist adds to it), the
+// lengths of the two lists of k_hot_lists (zero too), and the lists.
+struct HotScratch {
+    unsigned int* hist;
+    int *na, *nb, *la, *lb;
+    static constexpr int kZero = kHotBins + 2;  // words to be zeroed, from hist on
+    static __host__ __device__ constexpr size_t bytes(int cap) { return (size_t)(kZero + 2 * cap) * 4; }
+    __host__ HotScratch(void* p, int cap) {
+        hist = static_cast<unsigned int*>(p);
+        na = reinterpret_cast<int*>(hist + kHotBins);
+        nb = na + 1;
+        la = nb + 1;
+        lb = la + cap;
+    }
 };
 
-// Histogram of the out-degrees (those of kHotBins - 1 and more together).
+// (Not in k_row_scale, whose loop it slows by more than it takes: 4 M nodes,
+// 57 us there and 17 here against 102.)
 __global__ void __launch_bounds__(1024) k_degree_hist(const int* __restrict__ deg, int n, unsigned int* hist) {
     __shared__ unsigned int h[kHotBins];
     for (int b = threadIdx.x; b < kHotBins; b += blockDim.x) h[b] = 0u;
@@ -923,11 +935,11 @@ __global__ void __launch_bounds__(1024) k_degree_hist(const int* __restrict__ de
 // The hot sources (1024 threads): as many of the largest out-degrees as fit
 // `cap`, whole degrees only, none below kHotMinDegree. Hot nodes with ids
 // beyond their number go to list b, the others with smaller ids to list a
-// (equally many); every node's rank starts as its id.
-__global__ void __launch_bounds__(1024) k_hot_lists(const int* __restrict__ deg, int n,
-                                                    const unsigned int* __restrict__ hist, int cap, HotInfo* info,
-                                                    int* __restrict__ rank, int* __restrict__ la,
-                                                    int* __restrict__ lb) {
+// (equally many); every node's rank starts as its id, and x takes s in that
+// order.
+__global__ void __launch_bounds__(1024) k_hot_lists(const int* __restrict__ deg, int n, HotScratch h, int cap,
+                                                    int* __restrict__ n_hot, int* __restrict__ rank,
+                                                    const double* __restrict__ s, double* __restrict__ x) {
     __shared__ int s_thr, s_count;
     if (threadIdx.x == 0) {
         s_thr = 0x7fffffff;
@@ -936,17 +948,17 @@ __global__ void __launch_bounds__(1024) k_hot_lists(const int* __restrict__ deg,
     constexpr int kPer = kHotBins / 1024;
     unsigned long long mine = 0;
     const int top = kHotBins - 1 - (int)threadIdx.x * kPer;  // this thread's bins top, top - 1, ...
-    unsigned int h[kPer];
+    unsigned int hb[kPer];
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-        h[q] = hist[top - q];
-        mine += h[q];
+        hb[q] = h.hist[top - q];
+        mine += hb[q];
     }
     unsigned long long total;
     unsigned long long cum = block_exscan<1024>(mine, &total);
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-        cum += h[q];
+        cum += hb[q];
         // (the lowest bin that still fits; the count only grows downwards)
         if (top - q >= kHotMinDegree && cum <= (unsigned long long)cap) {
             atomicMin(&s_thr, top - q);
@@ -955,32 +967,27 @@ __global__ void __launch_bounds__(1024) k_hot_lists(const int* __restrict__ deg,
     }
     __syncthreads();
     const int thr = s_thr, count = s_count;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        info->thr = thr;
-        info->count = count;
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_hot = count;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         rank[i] = i;
+        x[i] = s[i];
         const bool hot = deg[i] >= thr;
-        if (hot && i >= count) lb[atomicAdd(&info->nb, 1)] = i;
-        if (!hot && i < count) la[atomicAdd(&info->na, 1)] = i;
+        if (hot && i >= count) h.lb[atomicAdd(h.nb, 1)] = i;
+        if (!hot && i < count) h.la[atomicAdd(h.na, 1)] = i;
     }
 }
 
-__global__ void k_hot_swap(const HotInfo* __restrict__ info, const int* __restrict__ la, const int* __restrict__ lb,
-                           int* __restrict__ rank) {
-    const int m = info->na;
+// The nodes of the two lists change places, in rank and in x.
+__global__ void k_hot_swap(HotScratch h, int* __restrict__ rank, double* __restrict__ x) {
+    const int m = *h.na;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-        rank[la[k]] = lb[k];
-        rank[lb[k]] = la[k];
+        const int a = h.la[k], b = h.lb[k];
+        rank[a] = b;
+        rank[b] = a;
+        const double xa = x[a];
+        x[a] = x[b];
+        x[b] = xa;
     }
-}
-
-// out[rank[i]] = x[i].
-__global__ void k_to_source_order(const double* __restrict__ x, const int* __restrict__ rank, int n,
-                                  double* __restrict__ out) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        out[source_of(rank, i)] = x[i];
 }
 
 // m~_i = m_i s_i, the cash a green row sends per unit of edge weight: in
@@ -1853,9 +1860,11 @@ __global__ void k_from_double(const double* __restrict__ x, int n, T* __restrict
 // row_ptr, 2 empty row, 4 col out of range, 8 bad weight.
 __global__ void k_validate(const long long* __restrict__ row_ptr, const int* __restrict__ col,
                            const float* __restrict__ w, long long n, long long nnz,
-                           unsigned int* err) {
+                           unsigned int* err, unsigned int* zero, int n_zero) {
     unsigned int e = 0;
     long long stride = (long long)gridDim.x * blockDim.x;
+    // (scratch that a later kernel adds to)
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_zero; i += stride) zero[i] = 0u;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += stride) {
         long long a = row_ptr[i], b = row_ptr[i + 1];
         if (b < a || a < 0 || b > nnz) e |= 1u;

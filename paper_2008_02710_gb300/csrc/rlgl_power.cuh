@@ -178,7 +178,7 @@ __device__ __forceinline__ T warp_segscan(K key, T val) {
 // L2) into shared memory; returns its length.
 template <typename T>
 __device__ __forceinline__ int load_hot(const SweepArgs<T>& A, const T* __restrict__ mt, PowSmem<T>& sm) {
-    const int n_hot = A.hot ? __ldg(&A.hot->count) : 0;
+    const int n_hot = A.n_hot ? __ldg(A.n_hot) : 0;
     if (threadIdx.x == 0) sm.next = kPowWarps;  // (every warp's first is its own)
     constexpr int kPer = 16 / (int)sizeof(T);
     const int nv = n_hot / kPer;

@@ -220,7 +220,7 @@ struct SweepArgs {
     int n_hubs;  // hub targets of the push, and the only one when there is one
     int hub1;
     const int* rank;  // source order of mt and mt2 (see source_of)
-    const HotInfo* hot;  // its hot front
+    const int* n_hot;  // length of its hot front
     T* mt;
     T* mt2;      // power sweep: the moved cash of every other move
     T* facc;     // power sweep: sums of rows split across tiles (zero at rest)
@@ -242,7 +242,6 @@ struct SweepArgs {
     unsigned long long cond_refresh;
     int use_cond;
     int n;
-    int vec_ok;
     const int* hubs;  // hub table of the push (nullptr: none)
 };
 
@@ -863,7 +862,6 @@ struct SweepCtl {
     SchedAux ax;       // this move's block-round-robin range and PC constants
     int have_lag;      // stale threshold: a move of this launch has set the statistics
     int stop;          // status to stop with now or after this move (-1: none)
-    int made;          // a move of this launch has been made
     int owed;          // block 0: the last move's state and log entry are still to be written
     MoveRecord rec;    // block 0: that entry (its times are in ts)
     double limit;      // links from which a move pulls
@@ -1072,7 +1070,7 @@ __device__ __forceinline__ void sweep_moves(const SweepArgs<T>& A) {
         sc.tk_pass = A.sw->bar.tk_pass;
         sc.limit = ctl.pull_crossover * (double)ctl.nnz;
         sc.l1 = sc.sumr = sc.mean = 0.0;
-        sc.have_lag = sc.leave = sc.made = sc.owed = sc.want_refresh = sc.tb = 0;
+        sc.have_lag = sc.leave = sc.owed = sc.want_refresh = sc.tb = 0;
         sc.stop = -1;
         sc.ts[0][0] = globaltimer();
         mv.mask = nullptr;
@@ -1125,7 +1123,6 @@ __device__ __forceinline__ void sweep_moves(const SweepArgs<T>& A) {
             sc.sumr = sumr;
             sc.mean = sumr / (double)n;
         }
-        sc.made = 1;
         sc.hsum += sc.mm.x;
         sc.habs += sc.mm.y;
         sc.mabs = sc.mm.y;
