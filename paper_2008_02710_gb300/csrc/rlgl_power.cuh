@@ -44,13 +44,12 @@
 //   and the links' loads not kept in L1 and first to leave L2     71 / 2557
 //   no register spilled, two sums a node instead of four          71 / 2295
 //   tiles from a counter of the block, not of the GPU             71 / 2136
-// (the start of the second row on its own machine, the rest beside it). More
-// hot sources are slower: what shared memory takes is taken from L1, which
-// the loads in flight need (36864: 170 / 6690 us with the same merge as the
-// first row). A spilled register in the tile loop costs more than a larger
-// tile gives: 1024 threads at 64 registers 120 / 3880 us. A load from L2
-// into a register that a shared-memory load also writes waits for it: the
-// hot values are read first.
+// More hot sources are slower: what shared memory takes is taken from L1,
+// which the loads in flight need (36864: 170 / 6690 us with the same merge as
+// the first row). A spilled register in the tile loop costs more than a larger
+// tile gives: 1024 threads at 64 registers 120 / 3880 us. A load from L2 into
+// a register that a shared-memory load also writes waits for it: the hot
+// values are read first.
 // The moved cash alternates between two buffers (mt and the residual
 // source hsrc, free while no re-derivation runs). The per-move totals
 // rotate over three slots: the decision of move t reads slot q, move t adds
@@ -216,9 +215,10 @@ __device__ __forceinline__ void ld_over(double& v, const double* p, bool pred) {
 // one size, so that the blocks end together. With the last two rounds handed
 // out one at a time from a counter of the whole GPU, which 3648 warps asked:
 // symmetrised R-MAT 24, 60 moves, 137.7 ms against 128.1; weighted R-MAT of
-// 2 M nodes, 20 moves, 4.06 against 3.89; R-MAT 20 4.32 against 4.34. While a warp sums a tile, the next tile's bounds and in-link
-// sources are in flight. No block-wide barrier: a warp's lanes meet only at
-// __syncwarp. The pieces of rows that cross tile boundaries go into facc.
+// 2 M nodes, 20 moves, 4.06 against 3.89; R-MAT 20 4.32 against 4.34.
+// While a warp sums a tile, the next tile's bounds and in-link sources are in
+// flight. No block-wide barrier: a warp's lanes meet only at __syncwarp. The
+// pieces of rows that cross tile boundaries go into facc.
 template <typename T, bool kHasW>
 __device__ __forceinline__ void power_tiles(const SweepArgs<T>& A, const T* __restrict__ mt_cur,
                                             PowSmem<T>& sm, int n_hot, PowAcc<T>& acc) {

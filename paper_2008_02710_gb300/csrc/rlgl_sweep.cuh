@@ -25,7 +25,8 @@
 // 23 us as a kernel of their own on the same links); PageRank of an R-MAT
 // graph of 500000 nodes 63 -> 48 us; symmetrised R-MAT 24, a move 317 -> 293
 // us, and 234 us with what a move touches once a node or link first to leave
-// L2 and no degree loaded beside 1/d (select 156 -> 78, push 161 -> 156).
+// L2 and no degree loaded beside 1/d (select 156 -> 78, push 161 -> 156); 239
+// in the order of the nodes (see push_rows).
 // With the stale threshold (Control::theta_lag) a move after the first of a
 // launch has no stats phase and no first barrier: its select gathers the
 // statistics of the cash it reads, and the next move's threshold and
@@ -567,7 +568,8 @@ __device__ __forceinline__ void node_pass(const SweepArgs<T>& A, const MoveView<
             if (gm >> q & 1u) {
                 m[q] = C[q] * (scale_is_idg ? idg[q] : __ldg(scale + i));
                 // (unit weights: see push_rows)
-                if (kPass == PASS_SELECT) deg[q] = (kFar ? need_idg : scale_is_idg) ? degree_of(idg[q], A.deg + i) : __ldg(A.deg + i);
+                if (kPass == PASS_SELECT)
+                    deg[q] = (kFar ? need_idg : scale_is_idg) ? degree_of(idg[q], A.deg + i) : __ldg(A.deg + i);
             }
         }
 #pragma unroll
@@ -773,8 +775,8 @@ __device__ __forceinline__ void push_rows(const SweepArgs<T>& A, SweepSmem<T>& s
 }
 
 // The dense moved cash of a move that pulls though it was not expected to:
-// cleared (PASS 0), then set from the block's lists (after a barrier: other
-// blocks' nodes do not matter, but the pull reads all of them).
+// cleared, then set from the block's list (a grid barrier follows: the pull
+// reads all of it).
 template <typename T>
 __device__ __forceinline__ void dense_from_lists(const SweepArgs<T>& A, SweepSmem<T>& sm) {
     const OwnNodes<T> own(A.n);
