@@ -1405,13 +1405,28 @@ __global__ void __launch_bounds__(kThreads) k_push(
 // contiguous runs (equal keys are never separated by a different key).
 // Returns this thread's scan value; s_key/s_val then hold every thread's
 // key and scan value.
-template <typename TV, int kBT = kThreads>
+// (kGroups: the block is that many groups of kBT threads, each with its own
+// tiles and its own barrier.)
+template <int kBT, int kGroups>
+__device__ __forceinline__ int group_thread() {
+    return kGroups == 1 ? (int)threadIdx.x : (int)threadIdx.x % kBT;
+}
+template <int kBT, int kGroups>
+__device__ __forceinline__ void group_sync() {
+    if constexpr (kGroups == 1) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / kBT), "n"(kBT) : "memory");
+}
+
+template <typename TV, int kBT = kThreads, int kGroups = 1>
 __device__ __forceinline__ TV block_segscan(int key, TV val, int* s_key, TV* s_val) {
     constexpr int kW = kBT / 32;
     constexpr unsigned kWMask = kW >= 32 ? 0xffffffffu : ((1u << kW) - 1u);
-    __shared__ int w_key[kW];
-    __shared__ TV w_val[kW];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ int g_key[kGroups][kW];
+    __shared__ TV g_val[kGroups][kW];
+    const int tid = group_thread<kBT, kGroups>();
+    int* const w_key = g_key[kGroups == 1 ? 0 : threadIdx.x / kBT];
+    TV* const w_val = g_val[kGroups == 1 ? 0 : threadIdx.x / kBT];
+    const int lane = tid & 31, wid = tid >> 5;
     TV x = val;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1423,7 +1438,7 @@ __device__ __forceinline__ TV block_segscan(int key, TV val, int* s_key, TV* s_v
         w_key[wid] = key;
         w_val[wid] = x;
     }
-    __syncthreads();
+    group_sync<kBT, kGroups>();
     if (wid == 0 && lane < kW) {
         // the same scan over the warp tails
         int k = w_key[lane];
@@ -1436,11 +1451,11 @@ __device__ __forceinline__ TV block_segscan(int key, TV val, int* s_key, TV* s_v
         }
         w_val[lane] = v;
     }
-    __syncthreads();
+    group_sync<kBT, kGroups>();
     if (wid > 0 && w_key[wid - 1] == key) x += w_val[wid - 1];
-    s_key[threadIdx.x] = key;
-    s_val[threadIdx.x] = x;
-    __syncthreads();
+    s_key[tid] = key;
+    s_val[tid] = x;
+    group_sync<kBT, kGroups>();
     return x;
 }
 
@@ -1456,7 +1471,7 @@ __device__ __forceinline__ TV block_segscan(int key, TV val, int* s_key, TV* s_v
 // Shared memory of the merge-path tile loop.
 // Merge-path items per thread for a block of kBT threads: a tile is
 // kBT * mp_ipt(kBT) items (2048 for 256 threads).
-__host__ __device__ constexpr int mp_ipt(int kBT) { return kBT >= 1024 ? 2 : (kBT >= 512 ? 4 : kMpIpt); }
+__host__ __device__ constexpr int mp_ipt(int kBT) { return kBT >= 512 ? 4 : kMpIpt; }
 
 template <typename TV, int kBT = kThreads>
 struct PullSmem {
@@ -1475,7 +1490,7 @@ struct PullSmem {
 // comes back): a load-then-store per row end would put one dependent L2
 // round trip per row end on the thread, serialised over the rows a warp's
 // threads end at different steps of the merge.
-template <typename TV, typename TO, bool kHasW, bool kCg, int kBT = kThreads>
+template <typename TV, typename TO, bool kHasW, bool kCg, int kBT = kThreads, int kGroups = 1>
 __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __restrict__ src,
                                            const long long* __restrict__ t_ptr,
                                            const int* __restrict__ t_src,
@@ -1486,16 +1501,18 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
                                            unsigned long long* next = nullptr) {
     constexpr int kIpt = mp_ipt(kBT);  // merge items per thread: a tile is kBT * kIpt items
     const unsigned long long pol = stream_policy();
-    __shared__ long long s_tnext;
+    const int tid = group_thread<kBT, kGroups>();
+    __shared__ long long g_tnext[kGroups];
+    long long& s_tnext = g_tnext[kGroups == 1 ? 0 : threadIdx.x / kBT];
     long long b = first;
     if (next) {
-        if (threadIdx.x == 0) s_tnext = (long long)atomicAdd(next, 1ull);
-        __syncthreads();
+        if (tid == 0) s_tnext = (long long)atomicAdd(next, 1ull);
+        group_sync<kBT, kGroups>();
         b = s_tnext;
-        __syncthreads();
+        group_sync<kBT, kGroups>();
     }
     while (b < ntiles) {
-        if (next && threadIdx.x == 0) s_tnext = (long long)atomicAdd(next, 1ull);  // read below
+        if (next && tid == 0) s_tnext = (long long)atomicAdd(next, 1ull);  // read below
         const long long r0 = tile_r[b], e0 = tile_e[b];
         const int nrows = (int)(tile_r[b + 1] - r0);
         const int nedges = (int)(tile_e[b + 1] - e0);
@@ -1504,31 +1521,31 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
             float wv[kIpt];
 #pragma unroll
             for (int q = 0; q < kIpt; ++q) {
-                const int k = threadIdx.x + q * kBT;
+                const int k = tid + q * kBT;
                 sidx[q] = (k < nedges) ? ld_stream(t_src + e0 + k, pol) : -1;
                 if (kHasW) wv[q] = (k < nedges) ? ld_stream(t_w + e0 + k, pol) : 0.0f;
             }
             // (a tile seldom holds more rows than the block has threads)
             int re = 0;
-            if ((int)threadIdx.x < nrows) re = (int)(__ldg(t_ptr + r0 + 1 + threadIdx.x) - e0);
+            if (tid < nrows) re = (int)(__ldg(t_ptr + r0 + 1 + tid) - e0);
             TV v[kIpt];
 #pragma unroll
             for (int q = 0; q < kIpt; ++q) v[q] = (sidx[q] >= 0) ? ld_shared_data<kCg>(src + sidx[q]) : TV(0);
 #pragma unroll
             for (int q = 0; q < kIpt; ++q) {
-                const int k = threadIdx.x + q * kBT;
+                const int k = tid + q * kBT;
                 if (k < nedges) sm.val[k] = kHasW ? v[q] * (TV)wv[q] : v[q];
             }
-            if ((int)threadIdx.x < nrows) sm.end[threadIdx.x] = re;
-            for (int k = threadIdx.x + kBT; k < nrows; k += kBT) sm.end[k] = (int)(__ldg(t_ptr + r0 + 1 + k) - e0);
+            if (tid < nrows) sm.end[tid] = re;
+            for (int k = tid + kBT; k < nrows; k += kBT) sm.end[k] = (int)(__ldg(t_ptr + r0 + 1 + k) - e0);
         }
-        if (threadIdx.x == 0) {
+        if (tid == 0) {
             sm.end[nrows] = 0x7fffffff;
             sm.start0 = (int)(t_ptr[r0] - e0);
         }
-        __syncthreads();
+        group_sync<kBT, kGroups>();
         const int total = nrows + nedges;
-        const int d = threadIdx.x * kIpt;
+        const int d = tid * kIpt;
         // head piece: the end of a row begun by earlier threads (rowA);
         // tail piece: a row that continues past this thread (carry). Rows
         // are local to the tile.
@@ -1574,19 +1591,19 @@ __device__ __forceinline__ void pull_tiles(TO* __restrict__ out, const TV* __res
         }
         // Join the pieces: carry of thread t plus the carries of the threads
         // before it on the same row.
-        const TV run = block_segscan<TV, kBT>(rowB, accB, sm.ckey, sm.cval);
+        const TV run = block_segscan<TV, kBT, kGroups>(rowB, accB, sm.ckey, sm.cval);
         if (rowA >= 0) {
             TV sum = accA;
-            if (threadIdx.x > 0 && sm.ckey[threadIdx.x - 1] == rowA) sum += sm.cval[threadIdx.x - 1];
+            if (tid > 0 && sm.ckey[tid - 1] == rowA) sum += sm.cval[tid - 1];
             red_add(out + (r0 + rowA), (TO)sum);
         }
         // last active thread: its carry leaves the tile
         const int last = (total - 1) / kIpt;
-        if ((int)threadIdx.x == last && rowB >= 0) red_add(out + (r0 + rowB), (TO)run);
-        __syncthreads();
+        if (tid == last && rowB >= 0) red_add(out + (r0 + rowB), (TO)run);
+        group_sync<kBT, kGroups>();
         if (next) {
             b = s_tnext;
-            __syncthreads();  // everyone has read s_tnext before thread 0 rewrites it
+            group_sync<kBT, kGroups>();  // everyone has read s_tnext before thread 0 rewrites it
         } else {
             b += step;
         }
